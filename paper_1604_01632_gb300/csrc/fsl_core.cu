@@ -67,7 +67,7 @@ __global__ void k_export_cells(const uint8_t* flag, const double* phi, const flo
     if (l >= n) return;
     const long long g = off + l;
     if (oflag) oflag[l] = ctype(flag[g]);
-    if (ophi) ophi[l] = phif ? (double)phif[g] : phi[g];
+    if (ophi) ophi[l] = phif ? to_double(phif[g]) : phi[g];
     if (om) om[l] = m[g];
     if (oid) {
         const int b = id[g];
