@@ -44,9 +44,47 @@ __host__ __device__ inline bool is_bubble_cell(uint8_t f) {
 
 __device__ inline int wrap1(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
 
-__global__ void k_static_init(const uint8_t* flags, int n, int* lab) {
+// Three kernels: runs, unions, labels.  All are bound by the latency of
+// dependent L2 accesses, not by their 9 B a cell, so the work is in shortening
+// the chains:
+//   - a cell starts on the first cell of its run along x inside its warp (one
+//     ballot) instead of on itself, which leaves about one root per warp and
+//     run and makes all unions along x inside a run unnecessary;
+//   - a cell unites with a neighbour row only where its left neighbour does not
+//     already do so (both left neighbours present means the same two runs);
+//   - the walk to a root halves the path behind it, and roots are hooked by
+//     compare-and-swap, so every cell points at an ancestor at all times.
+// 128^3 foam: 214 us with one union per cell and direction over unshortened
+// paths, 69 us in this form (host call included).
+
+__global__ void __launch_bounds__(256) k_static_init(const uint8_t* __restrict__ flags, int n, int nx,
+                                                     int* __restrict__ lab) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) lab[i] = is_bubble_cell(flags[i]) ? i : -1;   // every call starts from scratch
+    const bool fg = i < n && is_bubble_cell(flags[i]);
+    const unsigned m = __ballot_sync(0xffffffffu, fg);
+    if (i >= n) return;
+    if (!fg) { lab[i] = -1; return; }
+    // first cell of the run: after the last gap below this lane, not before the
+    // warp's first cell nor the row's
+    const int lane = threadIdx.x & 31;
+    const unsigned gaps = ~m & ((1u << lane) - 1u);
+    const int back = gaps ? lane - (32 - __clz((int)gaps)) : lane;
+    lab[i] = i - min(back, i % nx);
+}
+
+// Root of a, halving the path: a cell's parent only ever changes to an ancestor
+// (from itself to a smaller root, or to its grandparent), so a store, however
+// late, keeps the cell in its tree.
+__device__ inline int static_root_halving(int* L, int a) {
+    for (int it = 0; it < FSL_STATIC_MAX_CELLS; ++it) {
+        const int p = L[a];
+        if (p == a) return a;
+        const int gp = L[p];
+        if (gp == p) return p;
+        L[a] = gp;
+        a = gp;
+    }
+    return a;
 }
 
 __device__ inline int static_root(const int* L, int a) {
@@ -59,33 +97,55 @@ __device__ inline int static_root(const int* L, int a) {
     return a;
 }
 
-__global__ void k_static_hook(const uint8_t* flags, int nx, int ny, int nz, int* lab) {
+// Union: hook the larger root under the smaller while it is still a root; a
+// retry follows a link another thread made, so the loop ends.
+__device__ inline void static_unite(int* L, int a, int b) {
+    for (int it = 0; it < FSL_STATIC_MAX_CELLS; ++it) {
+        a = static_root_halving(L, a);
+        b = static_root_halving(L, b);
+        if (a == b) return;
+        if (a < b) { const int t = a; a = b; b = t; }
+        if (atomicCAS(&L[a], a, b) == a) return;
+    }
+}
+
+__global__ void __launch_bounds__(256) k_static_hook(const uint8_t* __restrict__ flags, int nx, int ny, int nz,
+                                                     int* __restrict__ lab) {
     const int n = nx * ny * nz;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n || !is_bubble_cell(flags[i])) return;
     const int x = i % nx, y = (i / nx) % ny, z = i / (nx * ny);
-    // one direction of each of the nine neighbour pairs of the 18-neighbourhood
-    const int d[9][3] = {{1, 0, 0}, {0, 1, 0}, {0, 0, 1}, {1, 1, 0}, {1, -1, 0},
-                         {1, 0, 1}, {1, 0, -1}, {0, 1, 1}, {0, 1, -1}};
-    for (int k = 0; k < 9; ++k) {
-        const int j = wrap1(x + d[k][0], nx) + nx * (wrap1(y + d[k][1], ny) + ny * wrap1(z + d[k][2], nz));
-        if (!is_bubble_cell(flags[j])) continue;
-        int a = i, b = j;
-        // union: hook the larger root under the smaller; a retry follows a link
-        // another thread made, so the loop ends
-        for (int it = 0; it < FSL_STATIC_MAX_CELLS; ++it) {
-            a = static_root(lab, a);
-            b = static_root(lab, b);
-            if (a == b) break;
-            if (a < b) { const int t = a; a = b; b = t; }
-            const int old = atomicMin(&lab[a], b);
-            if (old == a) break;
-            a = old;
-        }
-    }
+    const int row = i - x, xl = wrap1(x - 1, nx), xr = wrap1(x + 1, nx);
+    const int yp = nx * wrap1(y + 1, ny), ym = nx * wrap1(y - 1, ny), y0 = nx * y;
+    const int zp = nx * ny * wrap1(z + 1, nz), z0 = nx * ny * z;
+    // the rows of the nine neighbour pairs' second cells: +y, +z (with their x
+    // neighbours), +y+z and -y+z (straight only); every type loaded up front
+    const int ry = z0 + yp, rz = zp + y0, rd = zp + yp, ru = zp + ym;
+    const bool left_w = is_bubble_cell(flags[row + xl]), right = is_bubble_cell(flags[row + xr]);
+    const bool yl = is_bubble_cell(flags[ry + xl]), yc = is_bubble_cell(flags[ry + x]), yr = is_bubble_cell(flags[ry + xr]);
+    const bool zl = is_bubble_cell(flags[rz + xl]), zc = is_bubble_cell(flags[rz + x]), zr = is_bubble_cell(flags[rz + xr]);
+    const bool dl = is_bubble_cell(flags[rd + xl]), dc = is_bubble_cell(flags[rd + x]);
+    const bool ul = is_bubble_cell(flags[ru + xl]), uc = is_bubble_cell(flags[ru + x]);
+    // along x: only where a run goes on past its warp or the row's end
+    if (right && lab[row + xr] != lab[i] && (((threadIdx.x & 31) == 31) || xr != x + 1))
+        static_unite(lab, i, row + xr);
+    // straight neighbour: the left cells make the same union when both are there
+    // (never past the row's start, or a full row would leave it to itself)
+    const bool left = left_w && x > 0;
+    if (yc && !(left && yl)) static_unite(lab, i, ry + x);
+    if (zc && !(left && zl)) static_unite(lab, i, rz + x);
+    if (dc && !(left && dl)) static_unite(lab, i, rd + x);
+    if (uc && !(left && ul)) static_unite(lab, i, ru + x);
+    // diagonal neighbour: only where no straight union leads there (the cell
+    // below it, or this cell's neighbour on that side, would)
+    if (yr && !yc && !right) static_unite(lab, i, ry + xr);
+    if (yl && !yc && !left_w) static_unite(lab, i, ry + xl);
+    if (zr && !zc && !right) static_unite(lab, i, rz + xr);
+    if (zl && !zc && !left_w) static_unite(lab, i, rz + xl);
 }
 
-__global__ void k_static_out(const uint8_t* flags, int n, const int* lab, int64_t* out) {
+__global__ void __launch_bounds__(256) k_static_out(const uint8_t* __restrict__ flags, int n,
+                                                    const int* __restrict__ lab, int64_t* __restrict__ out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     out[i] = is_bubble_cell(flags[i]) ? (int64_t)static_root(lab, i) : -1;
@@ -113,7 +173,7 @@ extern "C" fsl_status fsl_label_bubbles_static(const uint8_t* flags, int32_t nx,
     int* lab = (int*)lab_ptr;
     cudaStream_t s = (cudaStream_t)cuda_stream;
     const int nb = (int)((n + 255) / 256);
-    k_static_init<<<nb, 256, 0, s>>>(flags, (int)n, lab);
+    k_static_init<<<nb, 256, 0, s>>>(flags, (int)n, nx, lab);
     k_static_hook<<<nb, 256, 0, s>>>(flags, nx, ny, nz, lab);
     k_static_out<<<nb, 256, 0, s>>>(flags, (int)n, lab, labels);
     return cudaGetLastError() == cudaSuccess ? FSL_OK : FSL_ERR_CUDA;
