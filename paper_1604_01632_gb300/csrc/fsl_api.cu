@@ -572,7 +572,8 @@ fsl_status fsl_create(const fsl_params* params, int32_t n_domains, int32_t preci
         D.feps = (float)D.eps;
         div_magic(p.nx, D.mgx, D.shx);
         div_magic(p.ny, D.mgy, D.shy);
-        D.has_force = (p.gravity[0] != 0.0 || p.gravity[1] != 0.0 || p.gravity[2] != 0.0) ? 1 : 0;
+        // F_NONE, F_ANY or F_Z (the FP64 kernels drop the terms of the zero components)
+        D.has_force = (p.gravity[0] != 0.0 || p.gravity[1] != 0.0) ? F_ANY : (p.gravity[2] != 0.0 ? F_Z : F_NONE);
         D.lonely_rule = p.lonely_rule;
         D.split_trigger = p.split_trigger;
         h->hdoms.push_back(D);
