@@ -1182,10 +1182,12 @@ __device__ inline void step_counters(const StepArgs& A) {
     for (int d = threadIdx.x; d < A.ndom; d += blockDim.x) {
         if (A.nif[d] > 0) A.pool[d] = 0;   // the pool was shared out last step
         A.nif[d] = A.icnt[d];
+        A.icnt[d] = 0;
         A.trig[1 + d] = 0;
     }
     if (threadIdx.x == 0) {
         *A.stepno += 1;
+        *A.icount_next = 0;
         *A.gcount = 0;
         *A.lcount = 0;
         *A.trig = 0;
@@ -2090,9 +2092,6 @@ __global__ void __launch_bounds__(FSL_BLOCK, sizeof(T) == 8 ? 2 : FSL_STREAM_MIN
 enum { SC_SPLIT = 0, SC_PERS1 = 1, SC_PERS2 = 2, SC_PERS4 = 3, SC_SLAB = 4, SC_TWO = 5, SC_TILE2 = 6, SC_TILE4 = 7,
        SC_TWOC = 8, SC_FORMS = 9 };
 
-// First neighbour of cell z (direction order) that is an interface cell
-// carrying mark `want`, or -1.
-//
 // The neighbour scans below load all eighteen neighbours first and then test
 // them (one memory latency, not one per neighbour): bit a of the mask is set
 // when neighbour a (1-18) is an interface cell carrying mark `want`.
@@ -2109,14 +2108,6 @@ __device__ inline unsigned marked_mask(const StepArgs& A, const Cell& c, uint8_t
     for (int a = 1; a < 19; ++a) m |= (unsigned)(ctype(fl[a]) == IFC && mk[a] == want) << a;
     return m;
 }
-__device__ inline long long first_marked(const StepArgs& A, const Dom& D, long long z, uint8_t want) {
-    const Cell c = make_cell(D, z);
-    const unsigned m = marked_mask(A, c, want);
-    if (m == 0) return -1;
-    const int a = __ffs(m) - 1;
-    return c.at(rcx(a), rcy(a), rcz(a));
-}
-
 // An interface cell carrying an emptied mark that phase A does not cancel (no
 // filled neighbour).  Written as a test on the marks the interface kernel
 // set, so it holds whether or not another thread has already cleared the
@@ -2128,22 +2119,23 @@ __device__ inline bool still_emptied(const StepArgs& A, const Dom& D, long long 
 }
 
 // Conversion phases A and B (Sec. 2.2, cell conversion), one thread per
-// (marked cell, direction).  A filled cell turns the gas neighbour in that
-// direction into interface when it is that neighbour's first filled neighbour
-// in direction order (so each new cell is claimed once) and initialises it
-// with f = f_eq of the mean density and velocity of its liquid and
-// non-emptied interface neighbours, m = 0; it also cancels an emptied mark
-// there.  An emptied cell with no filled neighbour turns the liquid neighbour
-// in that direction into interface when it is that neighbour's first such
-// emptied neighbour: the new cell keeps its PDFs, takes m = rho and joins the
-// emptied cell's bubble.
+// (marked cell, direction).  A filled cell claims the gas neighbour in that
+// direction (it becomes interface) when it is that neighbour's first filled
+// neighbour in direction order, so each new cell is claimed once; it also
+// cancels an emptied mark there.  An emptied cell with no filled neighbour
+// turns the liquid neighbour in that direction into interface when it is that
+// neighbour's first such emptied neighbour: the new cell keeps its PDFs, takes
+// m = rho and joins the emptied cell's bubble.  (The PDFs of the cells claimed
+// from gas are formed in phase C, where nothing waits for them.)
+//
+// A step marks few cells, so the phase is bound by its chain of dependent
+// loads.  The neighbour's type, its eighteen neighbours' types and marks and
+// the cell's own mark are loaded together: two latencies after the list entry.
 template <typename T>
-__device__ inline void convert_ab_phase(const StepArgs& A) {
-    using C = typename Form<T>::C;
-    const int nm = *A.mcount;
+__device__ inline void convert_ab_phase(const StepArgs& A, int nm) {
     const int total = 18 * nm;
     const long long S = A.stride;
-    T* f = (T*)A.fdst;
+    const T* f = (const T*)A.fdst;
     const int stride = gridDim.x * blockDim.x;
     for (int base = blockIdx.x * blockDim.x; base < total; base += stride) {
         const int t = base + threadIdx.x;
@@ -2154,81 +2146,48 @@ __device__ inline void convert_ab_phase(const StepArgs& A) {
             const int a = 1 + t % 18;
             const int d = block_dom(A, p);
             const Dom& D = get_dom(A, d);
-            const uint8_t mp = A.mark[p];
             const Cell c = make_cell(D, p);
             z = c.at(rcx(a), rcy(a), rcz(a));
-            const uint8_t tz = ctype(A.flag[z]);
+            const Cell cz_ = make_cell(D, z);
+            const uint8_t mp = A.mark[p], tz = ctype(A.flag[z]), mz = A.mark[z];
+            // z's interface neighbours that carry a filled / an emptied mark
+            unsigned filled = 0, emptied = 0;
+            {
+                uint8_t fl[19], mk[19];
+#pragma unroll
+                for (int q = 1; q < 19; ++q) {
+                    const long long w = cz_.at(cx(q), cy(q), cz(q));
+                    fl[q] = A.flag[w];
+                    mk[q] = A.mark[w];
+                }
+#pragma unroll
+                for (int q = 1; q < 19; ++q) {
+                    filled |= (unsigned)(ctype(fl[q]) == IFC && mk[q] == MK_FILLED) << q;
+                    emptied |= (unsigned)(ctype(fl[q]) == IFC && mk[q] == MK_EMPTIED) << q;
+                }
+            }
             if (mp == MK_FILLED) {
                 if (tz == GAS) {
-                    if (first_marked(A, D, z, MK_FILLED) == p) {
+                    // p is z's neighbour in the opposite direction
+                    if (__ffs(filled) - 1 == opp(a)) {
                         gclaim = true;
-                        // f = f_eq of the mean density and velocity of the liquid
-                        // and non-emptied interface neighbours, in direction order
-                        const Cell cz_ = make_cell(D, z);
-                        // which neighbours enter the mean: types and marks of all
-                        // eighteen first, the cancellation test only for the
-                        // emptied ones
-                        uint8_t fl[19], mk[19];
-#pragma unroll
-                        for (int q = 1; q < 19; ++q) {
-                            const long long w = cz_.at(cx(q), cy(q), cz(q));
-                            fl[q] = A.flag[w];
-                            mk[q] = A.mark[w];
-                        }
-                        unsigned use = 0, emp = 0;
-#pragma unroll
-                        for (int q = 1; q < 19; ++q) {
-                            const uint8_t tw = ctype(fl[q]);
-                            use |= (unsigned)(tw == LIQ || (tw == IFC && mk[q] != MK_EMPTIED)) << q;
-                            emp |= (unsigned)(tw == IFC && mk[q] == MK_EMPTIED) << q;
-                        }
-                        for (unsigned e = emp; e; e &= e - 1) {
-                            const int q = __ffs(e) - 1;
-                            if (!still_emptied(A, D, cz_.at(rcx(q), rcy(q), rcz(q)))) use |= 1u << q;
-                        }
-                        C sr = (C)0, sux = (C)0, suy = (C)0, suz = (C)0;
-                        int cnt = 0;
-                        for (int q = 1; q < 19; ++q) {
-                            const long long w = cz_.at(rcx(q), rcy(q), rcz(q));
-                            if ((use >> q) & 1u) {
-                                C fo[19];
-#pragma unroll
-                                for (int r = 0; r < 19; ++r) fo[r] = Form<T>::ld(f + (long long)r * S + w, r);
-                                C rr, jx, jy, jz;
-                                moments<C>(fo, rr, jx, jy, jz);
-                                sr = sr + rr;
-                                sux = sux + jx / rr;
-                                suy = suy + jy / rr;
-                                suz = suz + jz / rr;
-                                ++cnt;
-                            }
-                        }
-                        const C rbar = sr / (C)cnt;
-                        const C vx = sux / (C)cnt, vy = suy / (C)cnt, vz = suz / (C)cnt;
-                        C fe[19];
-                        feq_all<C>(rbar, vx, vy, vz, fe);
-#pragma unroll
-                        for (int r = 0; r < 19; ++r) Form<T>::st(f + (long long)r * S + z, r, fe[r]);
-                        A.m[z] = 0.0;
-                        A.rhoi[z] = (double)rbar;
                         A.mark[z] = MK_NEWG;
                         atomicAdd((unsigned long long*)&A.nif[d], 1ull);
                     }
-                } else if (tz == IFC && A.mark[z] == MK_EMPTIED) {
+                } else if (tz == IFC && mz == MK_EMPTIED) {
                     A.mark[z] = MK_NONE;
                 }
             } else if (mp == MK_EMPTIED && tz == LIQ && still_emptied(A, D, p)) {
                 // is p the first emptied-and-not-cancelled neighbour of z?
-                const Cell cz_ = make_cell(D, z);
-                long long first = -1;
-                for (unsigned e = marked_mask(A, cz_, MK_EMPTIED); e && first < 0; e &= e - 1) {
+                int first = -1;
+                for (unsigned e = emptied; e && first < 0; e &= e - 1) {
                     const int q = __ffs(e) - 1;
-                    const long long w = cz_.at(rcx(q), rcy(q), rcz(q));
-                    if (still_emptied(A, D, w)) first = w;
+                    if (q == opp(a) || still_emptied(A, D, cz_.at(rcx(q), rcy(q), rcz(q)))) first = q;
                 }
-                if (first == p) {
+                if (first == opp(a)) {
                     lclaim = true;
                     double r = (double)Form<T>::ld(f + z, 0);
+#pragma unroll
                     for (int q = 1; q < 19; ++q) r = r + (double)Form<T>::ld(f + (long long)q * S + z, q);
                     A.mark[z] = MK_NEWL;
                     A.id[z] = A.id[p];
@@ -2241,6 +2200,64 @@ __device__ inline void convert_ab_phase(const StepArgs& A) {
         }
         list_append(A.glist, A.gcount, gclaim, (int)z);
         list_append(A.llist, A.lcount, lclaim, (int)z);
+    }
+}
+
+// New interface cells from gas: f = f_eq of the mean density and velocity of
+// their liquid and non-emptied interface neighbours, m = 0.  One warp per cell,
+// lane q for the neighbour in direction q (its PDFs and moments), the means
+// summed in direction order.  One thread per cell walked up to eighteen
+// neighbours one after the other, nineteen loads and three divisions each, and
+// every other block waited for it at the next barrier (12-30 us a step on foams
+// of 2 M to 134 M cells, phases A and B with that barrier).
+template <typename T>
+__device__ inline void convert_newgas_phase(const StepArgs& A) {
+    using C = typename Form<T>::C;
+    const int ng = *A.gcount;
+    const long long S = A.stride;
+    T* f = (T*)A.fdst;
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int nw = (int)(gridDim.x * (blockDim.x >> 5));
+    // from the last warp down: the marked cells of phase C start at the first
+    for (int i = nw - 1 - (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); i < ng; i += nw) {
+        const long long z = A.glist[i];
+        const Dom& D = get_dom(A, block_dom(A, z));
+        const Cell c = make_cell(D, z);
+        bool use = false;
+        C r = (C)0, vx = (C)0, vy = (C)0, vz = (C)0;
+        if (lane >= 1 && lane < 19) {
+            const long long w = c.at(rcx(lane), rcy(lane), rcz(lane));
+            const uint8_t tw = ctype(A.flag[w]), mw = A.mark[w];
+            C fo[19];
+#pragma unroll
+            for (int q = 0; q < 19; ++q) fo[q] = Form<T>::ld(f + (long long)q * S + w, q);
+            // (phase C may already have renamed the mark of a converted cell)
+            use = tw == LIQ || (tw == IFC && mw != MK_EMPTIED && mw != MK_CEMPTIED);
+            if (use) {
+                C jx, jy, jz;
+                moments<C>(fo, r, jx, jy, jz);
+                vx = jx / r; vy = jy / r; vz = jz / r;
+            }
+        }
+        const unsigned um = __ballot_sync(full, use);
+        C sr = (C)0, sux = (C)0, suy = (C)0, suz = (C)0;
+        for (unsigned e = um; e; e &= e - 1) {
+            const int q = __ffs(e) - 1;
+            sr = sr + __shfl_sync(full, r, q);
+            sux = sux + __shfl_sync(full, vx, q);
+            suy = suy + __shfl_sync(full, vy, q);
+            suz = suz + __shfl_sync(full, vz, q);
+        }
+        const C cnt = (C)__popc(um);
+        const C rbar = sr / cnt;
+        C fe[19];
+        feq_all<C>(rbar, sux / cnt, suy / cnt, suz / cnt, fe);
+#pragma unroll
+        for (int q = 0; q < 19; ++q)
+            if (lane == q) Form<T>::st(f + (long long)q * S + z, q, fe[q]);
+        if (lane == 19) A.m[z] = 0.0;
+        if (lane == 20) A.rhoi[z] = (double)rbar;
     }
 }
 
@@ -2266,35 +2283,24 @@ __device__ inline void warp_add(long long* base, int key, long long v) {
 }
 
 // 3x3x3 cube around a cell, bit k = (dx+1) + 3 (dy+1) + 9 (dz+1); bit 13 is the
-// centre.  Face or edge neighbours of cube cell k inside the cube, the centre
-// left out (a walk must not pass through the removed cell).
-__host__ __device__ constexpr unsigned cube_adj18(int k) {
-    const int kx = k % 3 - 1, ky = (k / 3) % 3 - 1, kz = k / 9 - 1;
-    unsigned a = 0;
-    for (int j = 0; j < 27; ++j) {
-        const int ax = j % 3 - 1 - kx, ay = (j / 3) % 3 - 1 - ky, az = j / 9 - 1 - kz;
-        if (ax < -1 || ax > 1 || ay < -1 || ay > 1 || az < -1 || az > 1) continue;
-        const int dist = (ax != 0) + (ay != 0) + (az != 0);
-        if (dist >= 1 && dist <= 2) a |= 1u << j;
-    }
-    return a & ~(1u << 13);
+// centre.  The cells of a set and their neighbours along one axis inside the
+// cube, by shifts (a table in constant memory serialised the lanes of a warp).
+__host__ __device__ constexpr unsigned cube_x0() { return 0x1249249u; }                 // dx = -1
+__host__ __device__ constexpr unsigned cube_y0() { return 0x7u | 0x7u << 9 | 0x7u << 18; }   // dy = -1
+__host__ __device__ constexpr unsigned cube_dx(unsigned r) {
+    return ((r & ~(cube_x0() << 2)) << 1) | ((r & ~cube_x0()) >> 1);
 }
-// the table, folded at compile time
-__constant__ static const unsigned c_cube_adj18[27] = {
-    cube_adj18(0),  cube_adj18(1),  cube_adj18(2),  cube_adj18(3),  cube_adj18(4),  cube_adj18(5),  cube_adj18(6),
-    cube_adj18(7),  cube_adj18(8),  cube_adj18(9),  cube_adj18(10), cube_adj18(11), cube_adj18(12), cube_adj18(13),
-    cube_adj18(14), cube_adj18(15), cube_adj18(16), cube_adj18(17), cube_adj18(18), cube_adj18(19), cube_adj18(20),
-    cube_adj18(21), cube_adj18(22), cube_adj18(23), cube_adj18(24), cube_adj18(25), cube_adj18(26)};
-
-// bits of the 18 face / edge neighbours of the centre
-__host__ __device__ constexpr unsigned cube_mask18() {
-    unsigned m = 0;
-    for (int k = 0; k < 27; ++k) {
-        const int dk = (k % 3 != 1) + ((k / 3) % 3 != 1) + (k / 9 != 1);
-        if (dk >= 1 && dk <= 2) m |= 1u << k;
-    }
-    return m;
+__host__ __device__ constexpr unsigned cube_dy(unsigned r) {
+    return ((r & ~(cube_y0() << 6)) << 3) | ((r & ~cube_y0()) >> 3);
 }
+__host__ __device__ constexpr unsigned cube_dz(unsigned r) { return ((r << 9) & 0x7ffffffu) | (r >> 9); }
+// all face and edge neighbours of a set
+__host__ __device__ constexpr unsigned cube_grow18(unsigned r) {
+    return cube_dx(r) | cube_dy(r) | cube_dz(r) | cube_dy(cube_dx(r)) | cube_dz(cube_dx(r)) | cube_dz(cube_dy(r));
+}
+// the 18 face / edge neighbours of the centre, and the bit of direction a
+__host__ __device__ constexpr unsigned cube_mask18() { return cube_grow18(1u << 13); }
+static_assert(cube_mask18() == 0x2ebdebau, "the 18 face and edge neighbours of the centre");
 
 // Local test that removing the filled cell at the centre of the cube cannot
 // split its bubble: the gas/interface cells among its 18 neighbours must stay
@@ -2305,14 +2311,8 @@ __device__ inline bool removal_is_local(unsigned fg) {
     if (targets == 0) return true;
     unsigned reach = targets & (~targets + 1u);   // lowest target
     for (int it = 0; it < 27; ++it) {
-        unsigned grow = reach;
-        unsigned r = reach;
-        while (r) {
-            const int k = __ffs(r) - 1;
-            r &= r - 1;
-            grow |= c_cube_adj18[k];
-        }
-        grow &= fg;
+        // a walk must not pass through the removed cell
+        const unsigned grow = reach | (cube_grow18(reach) & fg & ~(1u << 13));
         if (grow == reach) break;
         reach = grow;
     }
@@ -2522,8 +2522,8 @@ __device__ inline bool antiparallel_normals(const StepArgs& A, const Dom& D, con
 // triggers.  Taking the filled cells away one at a time in index order, each
 // removal must pass the local test with the lower-index filled cells already
 // gone and the higher-index ones still present, or the labelling runs.
-__device__ inline void convert_c_phase(const StepArgs& A, const CclArgs& K) {
-    const int nm = *A.mcount, nl = *A.lcount;
+__device__ inline void convert_c_phase(const StepArgs& A, const CclArgs& K, int nm) {
+    const int nl = *A.lcount;
     const int total = nm + nl;
     const int step = *A.stepno;
     const int stride = gridDim.x * blockDim.x;
@@ -2535,37 +2535,41 @@ __device__ inline void convert_c_phase(const StepArgs& A, const CclArgs& K) {
         const uint8_t mk = A.mark[g];
         if (i < nm) {
             if (mk != MK_FILLED && mk != MK_EMPTIED) continue;   // emptied mark cancelled in phase A
-            const double mex = (mk == MK_FILLED) ? A.m[g] - A.rhoi[g] : A.m[g];
-            uint8_t fl[19], mz[19];
+            const double mg = A.m[g], rg = A.rhoi[g];
+            // types and marks of the 26 neighbours, a plane of nine at a time:
+            // rcv = interface after conversion, fgm = still gas / interface, or
+            // filled in this step with a higher index
+            unsigned rcv = 0, fgm = 0;
 #pragma unroll
-            for (int a = 1; a < 19; ++a) {
-                const long long z = c.at(cx(a), cy(a), cz(a));
-                fl[a] = A.flag[z];
-                mz[a] = A.mark[z];
+            for (int dz = -1; dz <= 1; ++dz) {
+                uint8_t fl[9], mz[9];
+                bool later[9];
+#pragma unroll
+                for (int k = 0; k < 9; ++k) {
+                    const long long z = c.at(k % 3 - 1, k / 3 - 1, dz);
+                    fl[k] = ctype(A.flag[z]);
+                    mz[k] = A.mark[z];
+                    later[k] = z > g;
+                }
+#pragma unroll
+                for (int k = 0; k < 9; ++k) {
+                    const uint8_t nt = new_type(fl[k], mz[k]);
+                    const bool lf = fl[k] == IFC && (mz[k] == MK_FILLED || mz[k] == MK_CFILLED) && later[k];
+                    rcv |= (unsigned)(nt == IFC) << (k + 9 * (dz + 1));
+                    fgm |= (unsigned)(nt == GAS || nt == IFC || lf) << (k + 9 * (dz + 1));
+                }
             }
-            unsigned rcv = 0;
-#pragma unroll
-            for (int a = 1; a < 19; ++a) rcv |= (unsigned)(new_type(ctype(fl[a]), mz[a]) == IFC) << a;
+            fgm &= ~(1u << 13);
+            rcv &= cube_mask18();
             const int k = __popc(rcv);
             for (unsigned e = rcv; e; e &= e - 1) {
-                const int a = __ffs(e) - 1;
-                A.recv[c.at(rcx(a), rcy(a), rcz(a))] = step;   // pulls a share in phase D
+                const int q = __ffs(e) - 1;
+                A.recv[c.at(q % 3 - 1, (q / 3) % 3 - 1, q / 9 - 1)] = step;   // pulls a share in phase D
             }
+            const double mex = (mk == MK_FILLED) ? mg - rg : mg;
             if (k > 0) A.exs[g] = mex / (double)k;
             else atomicAdd((unsigned long long*)&A.pool[d], (unsigned long long)__double2ll_rn(mex * 1099511627776.0));
             if (mk == MK_FILLED) {
-                unsigned fgm = 0;
-                for (int dz = -1; dz <= 1; ++dz)
-                    for (int dy = -1; dy <= 1; ++dy)
-                        for (int dx = -1; dx <= 1; ++dx) {
-                            if (dx == 0 && dy == 0 && dz == 0) continue;
-                            const long long z = c.at(dx, dy, dz);
-                            const uint8_t tz = ctype(A.flag[z]), mz = A.mark[z];
-                            const uint8_t ntz = new_type(tz, mz);
-                            const bool later_filled = (tz == IFC && (mz == MK_FILLED || mz == MK_CFILLED) && z > g);
-                            if (ntz == GAS || ntz == IFC || later_filled)
-                                fgm |= 1u << ((dx + 1) + 3 * (dy + 1) + 9 * (dz + 1));
-                        }
                 const bool may_split = D.split_trigger ? antiparallel_normals(A, D, c, g, A.id[g])
                                                        : !removal_is_local(fgm);
                 if (may_split) mark_affected(A, K, d, A.id[g]);   // its bubble may split
@@ -3137,19 +3141,23 @@ __device__ inline bool grid_barrier(const StepArgs& A) {
 template <typename T>
 __global__ void __launch_bounds__(FSL_CONV_THREADS, 3) k_convert(StepArgs A, CclArgs K) {
     pdl_wait();   // the stream-collide kernel has finished and its writes are visible
-    if (blockIdx.x == 0) {
-        for (int d = threadIdx.x; d < A.ndom; d += blockDim.x) A.icnt[d] = 0;
-        if (threadIdx.x == 0) {
-            *A.icount_next = 0;
-            // list counters of this step's labelling (used after phase C at the earliest)
-            *K.naff = 0; *K.np = 0; *K.nnew = 0; *K.nhused = 0;
-        }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        // list counters of this step's labelling (used after phase C at the earliest)
+        *K.naff = 0; *K.np = 0; *K.nnew = 0; *K.nhused = 0;
     }
-    convert_ab_phase<T>(A);
-    if (!grid_barrier(A)) return;
-    convert_c_phase(A, K);
-    if (!grid_barrier(A)) return;
-    const bool relabel = *(volatile int*)A.trig != 0;   // final after phase C
+    // no cell filled or emptied (the usual step of a quiet lattice): phases A to
+    // C have nothing to do, and phase D needs no barrier before it (5 us of the
+    // kernel's 10 us on a 32^3 lattice)
+    const int nm = *A.mcount;
+    bool relabel = false;
+    if (nm > 0 || A.bar_extra) {
+        convert_ab_phase<T>(A, nm);
+        if (!grid_barrier(A)) return;
+        convert_c_phase(A, K, nm);
+        convert_newgas_phase<T>(A);
+        if (!grid_barrier(A)) return;
+        relabel = *(volatile int*)A.trig != 0;   // final after phase C
+    }
     convert_d_phase(A);
     if (A.order) {
         if (!grid_barrier(A)) return;
