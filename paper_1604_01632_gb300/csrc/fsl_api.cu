@@ -91,10 +91,13 @@ struct fsl_domain {
     void* f[2] = {nullptr, nullptr};
     int cur = 0;
     uint8_t *flag = nullptr, *mark = nullptr;
-    double *m = nullptr, *phi = nullptr, *phit = nullptr, *rhoi = nullptr, *exs = nullptr;
-    float *phif = nullptr, *phitf = nullptr;   // FP32 copies (FP32-collide forms only)
+    double *m = nullptr, *exs = nullptr;
+    // interface cells, in the arithmetic type: fill level (one array per PDF
+    // buffer), stencil fill level, density
+    void *phi[2] = {nullptr, nullptr}, *phit = nullptr, *rhoi = nullptr;
+    bool list_ok = true;          // ilist[cur] holds the interface cells (the tile-fused forms keep none)
     void* nrm = nullptr;           // normals pass: 3 planes of the arithmetic type
-    unsigned* nmask = nullptr;     // normals pass: reconstruction directions per interface cell
+    unsigned long long* links = nullptr;   // normals pass: link word per interface cell
     void* pvc = nullptr;           // normals pass: bubble pressure per interface cell
     int* id = nullptr;
     long long *vfx = nullptr, *vxfx = nullptr, *vsfx = nullptr, *ncells = nullptr;
@@ -107,6 +110,7 @@ struct fsl_domain {
     int* icount[2] = {nullptr, nullptr};
     int *mlist = nullptr, *mcount = nullptr, *glist = nullptr, *gcount = nullptr, *llist = nullptr, *lcount = nullptr;
     int *cstep = nullptr, *recv = nullptr, *stepno = nullptr;
+    int *rlist = nullptr, *rcount = nullptr, *pflag = nullptr;
     long long* icnt = nullptr;
     // labelling scratch
     int *lab = nullptr, *aux = nullptr;
@@ -224,7 +228,18 @@ int order_effective(const fsl_domain* h) {
     return h->l2bytes > 0 && pdf_bytes > 2.0 * (double)h->l2bytes ? 1 : 0;
 }
 
-StepArgs step_args(fsl_domain* h, int src) {
+bool f64_form(const fsl_domain* h) { return h->precision == FSL_P_FP64; }
+
+bool tile_form(int f) { return f == SC_TILE2 || f == SC_TILE4; }
+
+// Whether steps of form f leave an interface list behind: the tile-fused forms
+// find their cells themselves, so only the tuning (which runs other forms next)
+// needs one after them.
+bool keeps_list(const fsl_domain* h, int f) { return !tile_form(f) || h->tuning; }
+
+// form: the stream-collide form of the step (-1: the handle's)
+StepArgs step_args(fsl_domain* h, int src, int form = -1) {
+    if (form < 0) form = h->form;
     StepArgs A;
     A.doms = h->d_doms;
     A.blk_dom = h->d_blk_dom;
@@ -236,13 +251,12 @@ StepArgs step_args(fsl_domain* h, int src) {
     A.flag = h->flag;
     A.mark = h->mark;
     A.m = h->m;
-    A.phi = h->phi;
+    A.phi = h->phi[src];
+    A.phi_next = h->phi[1 - src];
     A.phit = h->phit;
-    A.phif = h->phif;
-    A.phitf = h->phitf;
     A.bbox = h->bbox;
     A.nrm = h->nrm;
-    A.nmask = h->nmask;
+    A.links = h->links;
     A.pvc = h->pvc;
     A.rhoi = h->rhoi;
     A.exs = h->exs;
@@ -257,7 +271,12 @@ StepArgs step_args(fsl_domain* h, int src) {
     A.trig = h->trig;
     A.status = h->status;
     A.bar = h->bar;
-    A.order = order_effective(h);
+    // Fill levels in the interface kernel: in the forms that take interface
+    // cells one per thread, unless phase D has to walk the list anyway to append
+    // the next one (two-kernel forms with the list in appended order).
+    const int ord = order_effective(h);
+    A.fused = tile_form(form) || ((form == SC_TWO || form == SC_TWOC) && ord) ? 1 : 0;
+    A.order = tile_form(form) ? (keeps_list(h, form) ? 1 : 0) : ord;
     A.ocnt = h->ocnt;
     A.spins = h->spins;
     A.bar_extra = h->bar_extra;
@@ -275,6 +294,9 @@ StepArgs step_args(fsl_domain* h, int src) {
     A.cstep = h->cstep;
     A.recv = h->recv;
     A.stepno = h->stepno;
+    A.rlist = h->rlist;
+    A.rcount = h->rcount;
+    A.pflag = h->pflag;
     A.icnt = h->icnt;
     A.d0 = h->hdoms[0];
     return A;
@@ -447,6 +469,27 @@ fsl_status latch(fsl_domain* h) {
     return FSL_OK;
 }
 
+// The interface list of the present state in cell order.
+fsl_status order_list(fsl_domain* h) {
+    StepArgs A = step_args(h, 1 - h->cur);   // ilist_next: the list of buffer cur
+    cudaError_t e;
+    switch (h->precision) {
+    case FSL_P_FP64: e = launch_order<double>(A, h->convblocks, h->ls); break;
+    case FSL_P_FP32: e = launch_order<float>(A, h->convblocks, h->ls); break;
+    case FSL_P_F16S: e = launch_order<__half>(A, h->convblocks, h->ls); break;
+    default: e = launch_order<__nv_bfloat16>(A, h->convblocks, h->ls); break;
+    }
+    if (e != cudaSuccess) return cuda_fail(h, e, "interface list");
+    h->launches += 1;
+    h->list_ok = true;
+    return FSL_OK;
+}
+
+// The next step (of any form while tuning) reads the interface list.
+fsl_status ensure_list(fsl_domain* h) {
+    return h->list_ok || !keeps_list(h, h->form) ? FSL_OK : order_list(h);
+}
+
 fsl_status ensure_initial(fsl_domain* h) {
     if (!h->need_initial_ccl) return FSL_OK;
     for (int d = 0; d < h->ndom; ++d)
@@ -466,12 +509,17 @@ fsl_status ensure_initial(fsl_domain* h) {
     CK(h, cudaMemsetAsync(h->vsfx, 0, 8 * NS, h->ls));
     CK(h, cudaMemsetAsync(h->ncells, 0, 8 * NS, h->ls));
     CK(h, cudaMemsetAsync(h->constp, 0, 4 * NS, h->ls));
-    h->launches += launch_ccl(A, ccl_args(h, 1), h->nblocks, h->ls);
+    h->launches += launch_ccl(A, ccl_args(h, 1), h->nblocks, f64_form(h), h->ls);
     CK(h, cudaMemsetAsync(h->icount[h->cur], 0, sizeof(int), h->ls));
     CK(h, cudaMemsetAsync(h->icnt, 0, 8 * (size_t)h->ndom, h->ls));
     launch_build_ilist(A, h->nblocks, h->ls);
     h->launches += 1;
     CK(h, cudaGetLastError());
+    h->list_ok = true;
+    if (order_effective(h)) {   // the appended order is arbitrary
+        fsl_status st = order_list(h);
+        if (st != FSL_OK) return st;
+    }
     h->need_initial_ccl = false;
     return FSL_OK;
 }
@@ -642,16 +690,14 @@ fsl_status fsl_create(const fsl_params* params, int32_t n_domains, int32_t preci
     AL(h->flag, N);
     AL(h->mark, N);
     AL(h->m, 8 * N);
-    AL(h->phi, 8 * N);
-    AL(h->phit, 8 * N);
-    if (precision != FSL_P_FP64) {
-        AL(h->phif, 4 * N);
-        AL(h->phitf, 4 * N);
-    }
+    const size_t cb = precision == FSL_P_FP64 ? 8 : 4;   // bytes of the arithmetic type
+    AL(h->phi[0], cb * N);
+    AL(h->phi[1], cb * N);
+    AL(h->phit, cb * N);
     AL(h->nrm, 3 * N * (precision == FSL_P_FP64 ? 8 : 4));
-    AL(h->nmask, 4 * N);
+    AL(h->links, 8 * N);
     AL(h->pvc, N * (precision == FSL_P_FP64 ? 8 : 4));
-    AL(h->rhoi, 8 * N);
+    AL(h->rhoi, cb * N);
     AL(h->exs, 8 * N);
     AL(h->id, 4 * N);
     AL(h->vfx, 8 * NS);
@@ -677,6 +723,9 @@ fsl_status fsl_create(const fsl_params* params, int32_t n_domains, int32_t preci
     AL(h->cstep, 4 * N);
     AL(h->recv, 4 * N);
     AL(h->stepno, sizeof(int));
+    AL(h->rlist, 4 * N);
+    AL(h->rcount, sizeof(int));
+    AL(h->pflag, sizeof(int));
     AL(h->icnt, 8 * n_domains);
 
     AL(h->lab, 4 * N);
@@ -738,15 +787,16 @@ fsl_status fsl_create(const fsl_params* params, int32_t n_domains, int32_t preci
     if (e == cudaSuccess) e = cudaMemset(h->mark, 0, N);
     if (e == cudaSuccess) e = cudaMemset(h->id, 0xff, 4 * N);
     if (e == cudaSuccess) e = cudaMemset(h->m, 0, 8 * N);
-    if (e == cudaSuccess) e = cudaMemset(h->phi, 0, 8 * N);
-    if (e == cudaSuccess) e = cudaMemset(h->phit, 0, 8 * N);
-    if (e == cudaSuccess && h->phif) e = cudaMemset(h->phif, 0, 4 * N);
-    if (e == cudaSuccess && h->phitf) e = cudaMemset(h->phitf, 0, 4 * N);
+    if (e == cudaSuccess) e = cudaMemset(h->phi[0], 0, cb * N);
+    if (e == cudaSuccess) e = cudaMemset(h->phi[1], 0, cb * N);
+    if (e == cudaSuccess) e = cudaMemset(h->phit, 0, cb * N);
     if (e == cudaSuccess) e = cudaMemset(h->nrm, 0, 3 * N * (precision == FSL_P_FP64 ? 8 : 4));
-    if (e == cudaSuccess) e = cudaMemset(h->nmask, 0, 4 * N);
+    if (e == cudaSuccess) e = cudaMemset(h->links, 0, 8 * N);
     if (e == cudaSuccess) e = cudaMemset(h->pvc, 0, N * (precision == FSL_P_FP64 ? 8 : 4));
     if (e == cudaSuccess) e = cudaMemset(h->bbox, 0, 6 * 4 * NS);
-    if (e == cudaSuccess) e = cudaMemset(h->rhoi, 0, 8 * N);
+    if (e == cudaSuccess) e = cudaMemset(h->rhoi, 0, cb * N);
+    if (e == cudaSuccess) e = cudaMemset(h->rcount, 0, sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(h->pflag, 0, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(h->exs, 0, 8 * N);
     if (e == cudaSuccess) e = cudaMemset(h->f[0], 0, 19 * N * h->fbytes);
     if (e == cudaSuccess) e = cudaMemset(h->f[1], 0, 19 * N * h->fbytes);
@@ -926,7 +976,7 @@ fsl_status tune_step(fsl_domain* h) {
         CK(h, cudaEventCreate(&h->tev[0]));
         CK(h, cudaEventCreate(&h->tev[1]));
     }
-    StepArgs A = step_args(h, h->cur);
+    StepArgs A = step_args(h, h->cur, f);
     CK(h, cudaEventRecord(h->tev[0], h->ls));
     launch_k1(h, A, h->ls, nullptr, nullptr, f);
     CK(h, cudaEventRecord(h->tev[1], h->ls));
@@ -964,6 +1014,8 @@ fsl_status fsl_step(fsl_domain* h, int64_t nsteps) {
     if (st != FSL_OK) return st;
     h->stepped = true;
     join_in(h);
+    st = ensure_list(h);
+    if (st != FSL_OK) return st;
     int64_t k = 0;
     // autotuning steps first (each a real step of the simulation)
     while (h->tuning && k < nsteps) {
@@ -979,6 +1031,7 @@ fsl_status fsl_step(fsl_domain* h, int64_t nsteps) {
     }
     nsteps -= k;
     k = 0;
+    h->list_ok = keeps_list(h, h->form);
     if (!h->graphs) {
         // direct launches
         for (; k < nsteps; ++k) {
@@ -1129,7 +1182,11 @@ int32_t fsl_stream_form(const fsl_domain* h) { return h ? h->form : -1; }
 fsl_status fsl_set_interface_order(fsl_domain* h, int32_t mode) {
     if (!h || mode < -1 || mode > 1) return fail(h, FSL_ERR_ARG, "bad interface-order mode");
     CK(h, cudaStreamSynchronize(h->ls));
+    const int before = order_effective(h);
     h->order_mode = mode;
+    // a list appended so far is put in order before the next step (the slab form
+    // searches it)
+    if (order_effective(h) && !before && !h->need_initial_ccl) h->list_ok = false;
     if (h->form == SC_SLAB && !order_effective(h)) h->form = SC_SPLIT;   // the slab form needs the order
     drop_graphs(h);
     return FSL_OK;
@@ -1254,7 +1311,7 @@ fsl_status fsl_fields(fsl_domain* h, int32_t d, uint32_t mask, void* const* dst,
             if (mask & (1u << bit)) dev[bit] = parts[m++];
     }
     if (mask & (FSL_F_FLAGS | FSL_F_FILL | FSL_F_MASS | FSL_F_ID)) {
-        launch_export_cells(h->flag, h->phi, h->phif, h->m, h->id, h->minidx, D.off, D.n, (uint8_t*)dev[0], (double*)dev[1],
+        launch_export_cells(h->flag, h->phi[h->cur], f64_form(h), h->m, h->id, h->minidx, D.off, D.n, (uint8_t*)dev[0], (double*)dev[1],
                             (double*)dev[2], (long long*)dev[3], nullptr, h->ls);
         h->launches += 1;
     }
@@ -1286,7 +1343,7 @@ fsl_status fsl_cell_counts(fsl_domain* h, int32_t d, int64_t* counts) {
     join_in(h);
     const Dom& D = h->hdoms[d];
     CK(h, cudaMemsetAsync(h->counts, 0, 64, h->ls));
-    launch_export_cells(h->flag, h->phi, h->phif, h->m, h->id, h->minidx, D.off, D.n, nullptr, nullptr, nullptr, nullptr,
+    launch_export_cells(h->flag, h->phi[h->cur], f64_form(h), h->m, h->id, h->minidx, D.off, D.n, nullptr, nullptr, nullptr, nullptr,
                         h->counts, h->ls);
     h->launches += 1;
     long long c[8];

@@ -35,7 +35,8 @@ __global__ void __launch_bounds__(FSL_BLOCK) k_build_ilist(StepArgs A) {
 __global__ void __launch_bounds__(FSL_BLOCK) k_ccl_init(StepArgs A, CclArgs K) { ccl_init_phase(A, K); }
 __global__ void __launch_bounds__(FSL_BLOCK) k_ccl_hook(StepArgs A, CclArgs K) { ccl_hook_phase(A, K); }
 __global__ void __launch_bounds__(FSL_BLOCK) k_ccl_compress(StepArgs A, CclArgs K) { ccl_compress_phase(A, K); }
-__global__ void __launch_bounds__(FSL_BLOCK) k_ccl_pairs(StepArgs A, CclArgs K) { ccl_pairs_phase(A, K); }
+template <typename C>
+__global__ void __launch_bounds__(FSL_BLOCK) k_ccl_pairs(StepArgs A, CclArgs K) { ccl_pairs_phase<C>(A, K); }
 __global__ void __launch_bounds__(FSL_BLOCK) k_ccl_install(StepArgs A, CclArgs K) { ccl_install_phase(A, K); }
 
 // ------------------------------------------------------------------ exports
@@ -50,11 +51,11 @@ __global__ void k_export_minid(const int* id, long long off, int n, int* minidx)
     if (b >= 0 && (int)(threadIdx.x & 31u) == __ffs(peers) - 1) atomicMin(&minidx[b], (int)l);
 }
 
-// Cell export; phif (the FP32-collide forms' fill level, null in FP64) takes the
-// place of phi where given.
-__global__ void k_export_cells(const uint8_t* flag, const double* phi, const float* phif, const double* m, const int* id,
-                               const int* minidx, long long off, int n, uint8_t* oflag, double* ophi, double* om,
-                               long long* oid, long long* counts) {
+// Cell export; phi in the arithmetic type C, stored for interface cells only.
+template <typename C>
+__global__ void k_export_cells(const uint8_t* flag, const C* phi, const double* m, const int* id, const int* minidx,
+                               long long off, int n, uint8_t* oflag, double* ophi, double* om, long long* oid,
+                               long long* counts) {
     const long long l = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (counts) {
         const int t = l < n ? (int)ctype(flag[off + l]) : -1;
@@ -66,8 +67,16 @@ __global__ void k_export_cells(const uint8_t* flag, const double* phi, const flo
     }
     if (l >= n) return;
     const long long g = off + l;
-    if (oflag) oflag[l] = ctype(flag[g]);
-    if (ophi) ophi[l] = phif ? to_double(phif[g]) : phi[g];
+    const uint8_t t = ctype(flag[g]);
+    if (oflag) oflag[l] = t;
+    if (ophi) {
+        double v = t == LIQ ? 1.0 : 0.0;
+        if (t == IFC) {
+            if constexpr (sizeof(C) == 8) v = phi[g];
+            else v = to_double(phi[g]);
+        }
+        ophi[l] = v;
+    }
     if (om) om[l] = m[g];
     if (oid) {
         const int b = id[g];
@@ -81,11 +90,12 @@ void launch_build_ilist(const StepArgs& A, long long nb, cudaStream_t s) { k_bui
 
 // Initial labelling (K.initial = 1): the list phases run over a grid of one
 // thread per cell, which covers the participant list whatever its length.
-int launch_ccl(const StepArgs& A, const CclArgs& K, long long nb, cudaStream_t s) {
+int launch_ccl(const StepArgs& A, const CclArgs& K, long long nb, bool f64, cudaStream_t s) {
     k_ccl_init<<<(unsigned)nb, FSL_BLOCK, 0, s>>>(A, K);
     k_ccl_hook<<<(unsigned)nb, FSL_BLOCK, 0, s>>>(A, K);
     k_ccl_compress<<<(unsigned)nb, FSL_BLOCK, 0, s>>>(A, K);
-    k_ccl_pairs<<<(unsigned)nb, FSL_BLOCK, 0, s>>>(A, K);
+    if (f64) k_ccl_pairs<double><<<(unsigned)nb, FSL_BLOCK, 0, s>>>(A, K);
+    else k_ccl_pairs<float><<<(unsigned)nb, FSL_BLOCK, 0, s>>>(A, K);
     k_ccl_install<<<(unsigned)nb, FSL_BLOCK, 0, s>>>(A, K);
     return 5;
 }
@@ -94,11 +104,16 @@ void launch_export_minid(const int* id, long long off, int n, int* minidx, cudaS
     k_export_minid<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(id, off, n, minidx);
 }
 
-void launch_export_cells(const uint8_t* flag, const double* phi, const float* phif, const double* m, const int* id,
+void launch_export_cells(const uint8_t* flag, const void* phi, bool f64, const double* m, const int* id,
                          const int* minidx, long long off, int n, uint8_t* oflag, double* ophi, double* om,
                          long long* oid, long long* counts, cudaStream_t s) {
-    k_export_cells<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(flag, phi, phif, m, id, minidx, off, n, oflag, ophi,
-                                                              om, oid, counts);
+    const unsigned nb = (unsigned)((n + 255) / 256);
+    if (f64)
+        k_export_cells<double><<<nb, 256, 0, s>>>(flag, (const double*)phi, m, id, minidx, off, n, oflag, ophi, om, oid,
+                                                  counts);
+    else
+        k_export_cells<float><<<nb, 256, 0, s>>>(flag, (const float*)phi, m, id, minidx, off, n, oflag, ophi, om, oid,
+                                                 counts);
 }
 
 }  // namespace fsl

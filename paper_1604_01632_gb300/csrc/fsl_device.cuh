@@ -117,12 +117,16 @@ struct StepArgs {
     uint8_t* flag;
     uint8_t* mark;
     double* m;                  // interface mass
-    double* phi;                // fill level
-    double* phit;               // fill level as the normal stencil reads it: walls and
+    // fill levels and densities of interface cells, in the arithmetic type
+    const void* phi;            // fill level after the previous step (interface cells only:
+                                // liquid is 1, everything else 0 whatever is stored)
+    void* phi_next;             // fill level after this step
+    void* phit;                 // fill level as the normal stencil reads it: walls and
                                 // liquid 1, gas 0, interface clamp(phi, 0, 1)
-    float* phif;                // FP32 copies of phi and phit for the FP32-collide
-    float* phitf;               // forms (null for the FP64 form)
-    double* rhoi;               // density of interface cells at their last collision
+    void* rhoi;                 // density of interface cells at their last collision
+    int fused;                  // 1: the interface kernel of this step also forms the fill levels
+                                // and volume terms, and the conversion's phase D takes only the
+                                // cells that a conversion touched
     double* exs;                // excess-mass share of converted cells
     int* id;                    // bubble slot of gas/interface cells, -1 elsewhere
     long long* vfx;             // bubble volume of the cells (slot)
@@ -147,11 +151,15 @@ struct StepArgs {
     int* lcount;
     int* cstep;                 // step number at which each cell was last converted
     int* recv;                  // step number at which each cell last received excess mass
+    int* rlist;                 // fused steps: interface cells that receive excess mass (phase C)
+    int* rcount;
+    int* pflag;                 // some domain has pooled excess mass to share out
     int* stepno;                // device step counter
     long long* icnt;            // per-domain interface count at the end of the step
     unsigned* bar;              // grid barrier of the conversion kernel: count, generation
     int order;                  // 1: the conversion kernel rebuilds the next interface list in
-                                // cell order (after phase D), 0: phase D appends it
+                                // cell order (after phase D), 0: phase D appends it (in a fused
+                                // step: no list is made)
     int* ocnt;                  // interface cells per conversion block (ordered rebuild)
     int spins;                  // polls a block waits at a grid barrier before it gives up
     int bar_extra;              // arrivals a barrier waits for beyond the grid (0; 1 only to
@@ -161,8 +169,7 @@ struct StepArgs {
                                 // all of its cells; a box spanning a periodic seam is the full axis
     void* nrm;                  // normals pass: unit normals of the cells that need one,
                                 // three planes of the arithmetic type (x, y, z), stride apart
-    unsigned* nmask;            // normals pass: per interface cell, bit a set when the
-                                // reconstruction's normal test holds for direction a
+    unsigned long long* links;  // normals pass: per interface cell, its link word (below)
     void* pvc;                  // normals pass: per interface cell, its bubble's pressure
                                 // p_V (Eq. 13) in the arithmetic type
     Dom d0;                     // domain 0, read from the parameter space when ndom == 1
@@ -793,6 +800,12 @@ __device__ inline long long volume_term_f(uint8_t t, float phi) {
     return FSL_VOL_ONE - (long long)v;
 }
 
+// the same in the arithmetic type; and the fill level the normal stencil reads
+__device__ inline long long volume_term_c(uint8_t t, double phi) { return volume_term(t, phi); }
+__device__ inline long long volume_term_c(uint8_t t, float phi) { return volume_term_f(t, phi); }
+__device__ inline double clamp01(double v) { return v < 0.0 ? 0.0 : (v > 1.0 ? 1.0 : v); }
+__device__ inline float clamp01(float v) { return fminf(fmaxf(v, 0.f), 1.f); }
+
 __device__ inline uint8_t new_type(uint8_t t, uint8_t mk) {
     if (t == IFC) {
         if (mk == MK_FILLED || mk == MK_CFILLED) return LIQ;
@@ -1179,8 +1192,11 @@ __device__ inline void ph_row(int r, int& dy, int& dz) {
 // previous step's kernels are done with them; nothing in the stream-collide
 // kernel reads them).
 __device__ inline void step_counters(const StepArgs& A) {
+    if (threadIdx.x == 0) *A.pflag = 0;
+    __syncthreads();
     for (int d = threadIdx.x; d < A.ndom; d += blockDim.x) {
         if (A.nif[d] > 0) A.pool[d] = 0;   // the pool was shared out last step
+        else if (A.pool[d] != 0) *A.pflag = 1;
         A.nif[d] = A.icnt[d];
         A.icnt[d] = 0;
         A.trig[1 + d] = 0;
@@ -1190,6 +1206,7 @@ __device__ inline void step_counters(const StepArgs& A) {
         *A.icount_next = 0;
         *A.gcount = 0;
         *A.lcount = 0;
+        *A.rcount = 0;
         *A.trig = 0;
     }
 }
@@ -1204,11 +1221,9 @@ __device__ __forceinline__ void interface_chunk(const StepArgs& A, int i0, int c
     const unsigned S = (unsigned)A.stride;
     const T* __restrict__ src = (const T*)A.fsrc;
     T* __restrict__ dst = (T*)A.fdst;
-    // fill levels in the arithmetic type (FP32 copies for the FP32-collide forms)
-    const C* __restrict__ phic;
-    const C* __restrict__ phtc;
-    if constexpr (sizeof(C) == 8) { phic = A.phi; phtc = A.phit; }
-    else { phic = A.phif; phtc = A.phitf; }
+    // fill levels in the arithmetic type
+    const C* __restrict__ phic = (const C*)A.phi;
+    const C* __restrict__ phtc = (const C*)A.phit;
     const int c = threadIdx.x / TPC;      // cell of this thread in the load and gradient phases
     const int q = threadIdx.x % TPC;
     {
@@ -1443,7 +1458,7 @@ __device__ __forceinline__ void interface_chunk(const StepArgs& A, int i0, int c
                     }
                     const double mnew = sh.m[c] + (double)dm;
                     A.m[g] = mnew;
-                    A.rhoi[g] = (double)rho;
+                    ((C*)A.rhoi)[g] = rho;
                     bool filled, emptied;
                     if constexpr (sizeof(C) == 8) {
                         filled = mnew > (1.0 + D.eps) * rho;
@@ -1460,7 +1475,7 @@ __device__ __forceinline__ void interface_chunk(const StepArgs& A, int i0, int c
                         if (!has_gas) mk = MK_FILLED;
                         else if (!has_liq) mk = MK_EMPTIED;
                     }
-                    A.mark[g] = mk;
+                    if (mk != MK_NONE) A.mark[g] = mk;   // (it is MK_NONE between steps)
                 }
             }
             list_append(A.mlist, A.mcount, mk != MK_NONE, (int)g);
@@ -1503,12 +1518,26 @@ __device__ __forceinline__ void pyg_of(V&& v, C& gx, C& gy, C& gz) {
     }
 }
 
-// Stores of the normals pass for a cell g that needs a normal: the normal-test
-// bits of an interface cell, and the unit normal -grad/|grad| (0 where the
+// Link word of an interface cell, written by the normals pass (which has the
+// types of the cell's surroundings in shared memory) and read by the kernels
+// that take interface cells one per thread.  Per direction a: bit a - 1, the
+// reconstruction's normal test; bits 18 + 2 (a - 1), the kind of the source
+// x - c_a: 0 liquid, 1 interface, 2 gas, 3 wall.  Bit 54: some wall is a lid.
+// One 8-byte load takes the place of eighteen scattered type loads and their
+// addresses, and tells which of the other thirty-six neighbour loads (PDF, fill
+// level) have a use.
+constexpr unsigned long long LINK_LID = 1ull << 54;
+__device__ __forceinline__ unsigned long long link_kind(uint8_t t, int a) {
+    return (unsigned long long)(t < OBS ? t : OBS) << (16 + 2 * a);
+}
+
+// Stores of the normals pass for a cell g that needs a normal: the link word of
+// an interface cell (`kinds`: its types part), and the unit normal -grad/|grad| (0 where the
 // gradient is 0), with the arithmetic of the interface kernels (in FP64; the
 // FP32-collide forms scale by a reciprocal square root).
 template <typename C>
-__device__ __forceinline__ void normal_out(const StepArgs& A, unsigned g, bool ifc, C gx, C gy, C gz) {
+__device__ __forceinline__ void normal_out(const StepArgs& A, unsigned g, bool ifc, unsigned long long kinds, C gx, C gy,
+                                           C gz) {
     if (ifc) {
         // the bubble pressure the interface kernel would look up through the
         // cell's bubble (a load that waits on another): looked up here
@@ -1523,8 +1552,8 @@ __device__ __forceinline__ void normal_out(const StepArgs& A, unsigned g, bool i
         unsigned mk = 0;
 #pragma unroll
         for (int a = 1; a < 19; ++a)
-            mk |= (unsigned)(((C)cx(a) * gx + (C)cy(a) * gy) + (C)cz(a) * gz > (C)0) << a;
-        A.nmask[g] = mk;
+            mk |= (unsigned)(((C)cx(a) * gx + (C)cy(a) * gy) + (C)cz(a) * gz > (C)0) << (a - 1);
+        A.links[g] = kinds | mk;
     }
     C nx = gx, ny = gy, nz = gz;
     const C qq = nx * nx + ny * ny + nz * nz;
@@ -1547,6 +1576,17 @@ __device__ __forceinline__ void normal_out(const StepArgs& A, unsigned g, bool i
     nr[2u * S + g] = nz;
 }
 
+// The types part of the link word from the type array (the per-cell pass).
+__device__ inline unsigned long long link_kinds(const Pull& P, const uint8_t* flag) {
+    unsigned long long w = 0;
+#pragma unroll
+    for (int a = 1; a < 19; ++a) {
+        const uint8_t t = ctype(flag[P.at(-cx(a), -cy(a), -cz(a))]);
+        w |= link_kind(t, a) | (t == LID ? LINK_LID : 0ull);
+    }
+    return w;
+}
+
 // Normals pass, one thread per cell of the padded lattice, ahead of the
 // stream-collide kernels that take the interface cells one per thread.  The
 // curvature of an interface cell x (Eq. 15) is half the divergence of the unit
@@ -1554,8 +1594,8 @@ __device__ __forceinline__ void normal_out(const StepArgs& A, unsigned g, bool i
 // reconstruction's normal test (Eq. 11) uses the gradient at x itself.  Each
 // normal is computed here once, for every cell that is an interface cell or a
 // face neighbour of one (walls included: the stencil reads walls as full), and
-// stored in nrm; each interface cell also stores its 18 normal-test bits in
-// nmask, and the pressure of its bubble (Eq. 13) in pvc.  The stencil values
+// stored in nrm; each interface cell also stores its 18 link word in
+// links, and the pressure of its bubble (Eq. 13) in pvc.  The stencil values
 // are the stored copy phit (walls and liquid 1, gas 0, interface clamp(phi, 0,
 // 1)) and the arithmetic is that of the interface kernels, so their curvature
 // and reconstruction come out as if they had computed the normals themselves.
@@ -1572,9 +1612,7 @@ __global__ void __launch_bounds__(FSL_BLOCK) k_normals(StepArgs A) {
     using C = typename Form<T>::C;
     const long long g = (long long)blockIdx.x * FSL_BLOCK + threadIdx.x;   // stride: a multiple of the block
     const Dom& D = dom_at<ONE>(A, g);
-    const C* __restrict__ ph;
-    if constexpr (sizeof(C) == 8) ph = A.phit;
-    else ph = A.phitf;
+    const C* __restrict__ ph = (const C*)A.phit;
     const unsigned lane = threadIdx.x & 31u;
     const long long l0 = g - lane - D.off;   // the warp's first cell in its domain
     int x0, y, z;
@@ -1614,7 +1652,9 @@ __global__ void __launch_bounds__(FSL_BLOCK) k_normals(StepArgs A) {
         if (!need) return;
         C gx, gy, gz;
         pyg_of<C>([&](int dx, int dy, int dz) { return v[dz + 1][dy + 1][dx + 1]; }, gx, gy, gz);
-        normal_out<C>(A, gi, t == IFC, gx, gy, gz);
+        unsigned long long kinds = 0;
+        if (t == IFC) kinds = link_kinds(make_pull(D, g), A.flag);
+        normal_out<C>(A, gi, t == IFC, kinds, gx, gy, gz);
         return;
     }
     if (g - D.off >= D.n) return;   // padding after the domain
@@ -1628,7 +1668,9 @@ __global__ void __launch_bounds__(FSL_BLOCK) k_normals(StepArgs A) {
     if (!need) return;
     C gx, gy, gz;
     pyg_of<C>([&](int dx, int dy, int dz) { return ph[st.at(dx, dy, dz)]; }, gx, gy, gz);
-    normal_out<C>(A, (unsigned)g, t == IFC, gx, gy, gz);
+    unsigned long long kinds = 0;
+    if (t == IFC) kinds = link_kinds(make_pull(D, g), A.flag);
+    normal_out<C>(A, (unsigned)g, t == IFC, kinds, gx, gy, gz);
 }
 
 // The normals pass of a single-domain handle by 3D tiles: a block takes a
@@ -1664,9 +1706,7 @@ __global__ void __launch_bounds__(NT_X * NT_Y) k_normals_tiled(StepArgs A) {
         x0 = t.y; y0 = t.z; z0 = t.w;
     }
     const Dom& D = *Dp;
-    const C* __restrict__ ph;
-    if constexpr (sizeof(C) == 8) ph = A.phit;
-    else ph = A.phitf;
+    const C* __restrict__ ph = (const C*)A.phit;
     const unsigned off = (unsigned)D.off;
     // all loads of the thread first, then the shared stores (element i of the
     // halo tile is entry i of the flattened shared arrays)
@@ -1722,8 +1762,79 @@ __global__ void __launch_bounds__(NT_X * NT_Y) k_normals_tiled(StepArgs A) {
         const int hx = cx_ + 1, hy = cy_ + 1, hz = cz_ + 1;
         C gx, gy, gz;
         pyg_of<C>([&](int dx, int dy, int dz) { return vs[hz + dz][hy + dy][hx + dx]; }, gx, gy, gz);
-        normal_out<C>(A, off + (unsigned)((x0 + cx_) + D.nx * ((y0 + cy_) + D.ny * (z0 + cz_))),
-                      ts[hz][hy][hx] == IFC, gx, gy, gz);
+        const bool ifc = ts[hz][hy][hx] == IFC;
+        unsigned long long kinds = 0;
+        if (ifc) {
+#pragma unroll
+            for (int a = 1; a < 19; ++a) {
+                const uint8_t t = ts[hz - cz(a)][hy - cy(a)][hx - cx(a)];
+                kinds |= link_kind(t, a) | (t == LID ? LINK_LID : 0ull);
+            }
+        }
+        normal_out<C>(A, off + (unsigned)((x0 + cx_) + D.nx * ((y0 + cy_) + D.ny * (z0 + cz_))), ifc, kinds, gx, gy, gz);
+    }
+}
+
+// Sum v over the lanes of the warp that share a key into base[key], one
+// atomic per distinct key (the values are fixed point, so the order of the
+// additions does not matter); key < 0 contributes nothing.  Every lane of the
+// warp must call.
+__device__ inline void warp_add(long long* base, int key, long long v) {
+    const unsigned full = 0xffffffffu;
+    const int k0 = __shfl_sync(full, key, 0);
+    if (__all_sync(full, key == k0)) {
+        if (k0 < 0) return;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(full, v, o);
+        if ((threadIdx.x & 31) == 0 && v != 0) atomicAdd((unsigned long long*)&base[k0], (unsigned long long)v);
+        return;
+    }
+    const unsigned peers = __match_any_sync(full, key);
+    long long sum = 0;
+    for (unsigned m = peers; m; m &= m - 1) sum += __shfl_sync(peers, v, __ffs(m) - 1);
+    if ((int)(threadIdx.x & 31) == __ffs(peers) - 1 && key >= 0 && sum != 0)
+        atomicAdd((unsigned long long*)&base[key], (unsigned long long)sum);
+}
+
+// Rounding of f_eq,a + f_eq,abar = (fp + fm) + (fp - fm) in the FP32-collide
+// two-kernel forms.  fp = wr inn and fm = wr c3 are products, and which of them
+// is fused into its addition decides the last bit of a rebuilt PDF.  These forms
+// have one fixed choice per direction (and storage width, single domain or
+// batch, gas source or normal test), written out here so that a state does not
+// depend on how a compiler arranges the kernel around it:
+//   u  both products rounded first        p  fp fused in both sums
+//   m  fm fused in both sums              x  fm fused in the first, fp in the second
+// (The tile-fused forms take u for odd and p for even directions, FP64 u.)
+__host__ __device__ constexpr char two_kernel_rounding(int a, bool wide, bool one, bool gas) {
+    const char* t = wide ? (one ? (gas ? "uupupupuxpupupupup" : "uupupupuupupupupup")
+                                : (gas ? "pupuppmpppxpmmmpmp" : "pupuppupppupuuupmp"))
+                         : (one ? (gas ? "pupuuupuxpupupupup" : "pupuuupuupupupupup")
+                                : (gas ? "uuupuupppmxpupmpup" : "uuupuupppmupupupup"));
+    return t[a - 1];
+}
+template <char R>
+__device__ __forceinline__ float feq_both32(float wr, float inn, float c3) {
+    const float fp = __fmul_rn(wr, inn), fm = __fmul_rn(wr, c3);
+    float plus, minus;
+    if constexpr (R == 'u') { plus = __fadd_rn(fp, fm); minus = __fsub_rn(fp, fm); }
+    else if constexpr (R == 'p') { plus = __fmaf_rn(wr, inn, fm); minus = __fmaf_rn(wr, inn, -fm); }
+    else if constexpr (R == 'm') { plus = __fmaf_rn(wr, c3, fp); minus = __fmaf_rn(-wr, c3, fp); }
+    else { plus = __fmaf_rn(wr, c3, fp); minus = __fmaf_rn(wr, inn, -fm); }
+    return __fadd_rn(plus, minus);
+}
+// c_a . v without the zero terms, a odd
+template <int a>
+__device__ __forceinline__ float cdot32(float vx, float vy, float vz) {
+    constexpr int X = cx(a), Y = cy(a), Z = cz(a);
+    if constexpr (X != 0) {
+        if constexpr (Y != 0) return Y > 0 ? __fadd_rn(vx, vy) : __fsub_rn(vx, vy);
+        else if constexpr (Z != 0) return Z > 0 ? __fadd_rn(vx, vz) : __fsub_rn(vx, vz);
+        else return vx;
+    } else if constexpr (Y != 0) {
+        if constexpr (Z != 0) return Z > 0 ? __fadd_rn(vy, vz) : __fsub_rn(vy, vz);
+        else return vy;
+    } else {
+        return vz;
     }
 }
 
@@ -1733,35 +1844,55 @@ __global__ void __launch_bounds__(NT_X * NT_Y) k_normals_tiled(StepArgs A) {
 // links in direction order, Eq. 10; reconstruction from the bubble's gas
 // density 3 (p_V + 2 sigma kappa), Eqs. 8, 11-15; collision, Eq. 6; filled /
 // emptied marks).  The curvature and the normal test come from the normals
-// pass (k_normals), run before this kernel in the same step.  Returns whether
-// the cell was marked.
-template <typename T, bool ONE>
-__device__ __forceinline__ bool iface_one(const StepArgs& A, long long g) {
+// pass (k_normals), run before this kernel in the same step.
+//
+// In a fused step the cell also takes its new fill level phi = m / rho (Eq. 9)
+// here, where mass and density are in registers, and its bubble the difference
+// of the cell's volume term.  Before, phase D of the conversion did this for
+// every interface cell, reading and writing a dozen arrays a sector each
+// (0.57 ms of the 7.2 ms step of the 512^3 foam, 70 us of 1.28 ms at 256^3 FP32);
+// it now takes only converted cells, receivers of excess mass and new cells, and
+// corrects by differences from the value stored here.  Neighbours still read
+// this cell's old fill level, hence the two buffers.
+template <typename C> struct IfOut {
+    bool marked;
+    int key;          // fused step: bubble of the cell and change of its volume term
+    long long dv;
+};
+// TWO: the two-kernel forms (their rounding of the rebuilt PDFs, above).
+template <typename T, bool ONE, bool TWO>
+__device__ __forceinline__ IfOut<typename Form<T>::C> iface_one(const StepArgs& A, long long g) {
     using C = typename Form<T>::C;
     const Dom& D = dom_at<ONE>(A, g);
     const Par<C> R = par_of<C>(D);
-    const Stencil st = make_stencil(D, g);
     const unsigned S = (unsigned)A.stride;
     const T* __restrict__ src = (const T*)A.fsrc;
     T* __restrict__ dst = (T*)A.fdst;
-    const C* __restrict__ phic;
-    if constexpr (sizeof(C) == 8) phic = A.phi;
-    else phic = A.phif;
-    // own PDFs, and per direction a the source x - c_a: its type, the PDF
-    // streaming in and its fill level
-    // (the 18 source types packed 3 bits each: ty(a) = (tym >> 3a) & 7)
+    const C* __restrict__ phic = (const C*)A.phi;
+    const unsigned long long link = A.links[g];
+    const Pull P = make_pull(D, g);
+    auto at = [&](int dx, int dy, int dz) {
+        return (unsigned)g + (unsigned)(P.ox[dx + 1] + P.oy[dy + 1] + P.oz[dz + 1]);
+    };
+    // kind of the source x - c_a of direction a
+    auto ty = [&](int a) { return (uint8_t)((unsigned)(link >> (16 + 2 * a)) & 3u); };
+    auto is_lid = [&](int a) {
+        return (link & LINK_LID) && ctype(A.flag[at(-cx(a), -cy(a), -cz(a))]) == LID;
+    };
+    // own PDFs, and per direction a of the source x - c_a the PDF streaming in
+    // and the fill level, where the link has a use for them: a gas or wall source
+    // streams nothing in, and only interface neighbours weigh the mass exchange
     C fs[19], fy[19], phy[19];
-    unsigned long long tym = 0;
     fs[0] = Form<T>::ld(src + (unsigned)g, 0);
 #pragma unroll
     for (int a = 1; a < 19; ++a) {
         fs[a] = Form<T>::ld(src + ((unsigned)a * S + (unsigned)g), a);
-        const unsigned y = st.at(-cx(a), -cy(a), -cz(a));
-        tym |= (unsigned long long)ctype(A.flag[y]) << (3 * a);
-        fy[a] = Form<T>::ld(src + ((unsigned)a * S + y), a);
-        phy[a] = phic[y];
+        const unsigned y = at(-cx(a), -cy(a), -cz(a));
+        fy[a] = (C)0;
+        phy[a] = (C)0;
+        if (ty(a) <= IFC) fy[a] = Form<T>::ld(src + ((unsigned)a * S + y), a);
+        if (ty(a) == IFC) phy[a] = phic[y];
     }
-    auto ty = [&](int a) { return (uint8_t)((tym >> (3 * a)) & 7u); };
     const C phx = phic[g];
     const double m0 = A.m[g];
     const C pv = ((const C*)A.pvc)[g];   // the bubble's pressure, from the normals pass
@@ -1783,11 +1914,11 @@ __device__ __forceinline__ bool iface_one(const StepArgs& A, long long g) {
     // curvature (Eq. 15): half the divergence of the face neighbours' unit
     // normals by central differences; the normal test bits of the cell
     const C* __restrict__ nr = (const C*)A.nrm;
-    const C dX = nr[st.at(1, 0, 0)] - nr[st.at(-1, 0, 0)];
-    const C dY = nr[S + st.at(0, 1, 0)] - nr[S + st.at(0, -1, 0)];
-    const C dZ = nr[2u * S + st.at(0, 0, 1)] - nr[2u * S + st.at(0, 0, -1)];
+    const C dX = nr[at(1, 0, 0)] - nr[at(-1, 0, 0)];
+    const C dY = nr[S + at(0, 1, 0)] - nr[S + at(0, -1, 0)];
+    const C dZ = nr[2u * S + at(0, 0, 1)] - nr[2u * S + at(0, 0, -1)];
     const C kappa = (C)0.25 * ((dX + dY) + dZ);
-    const unsigned nmk = A.nmask[g];
+    const unsigned nmk = (unsigned)(link & 0x3ffffu) << 1;   // bit a: the normal test of direction a
     // gas velocity: that of the cell's own post-collision PDFs
     C rs, jsx, jsy, jsz;
     moments<C>(fs, rs, jsx, jsy, jsz);
@@ -1816,9 +1947,8 @@ __device__ __forceinline__ bool iface_one(const StepArgs& A, long long g) {
             const bool ra = rebuild(a), rb = rebuild(b);
             auto streamed = [&](int k, double own) {
                 const uint8_t t = ty(k);
-                if (t == OBS) return own;
-                if (t == LID) return own + (6.0 * weightc<C>(k)) * cdot<C>(k, R.lid[0], R.lid[1], R.lid[2]);
-                return fy[k];
+                if (t != OBS) return fy[k];
+                return is_lid(k) ? own + (6.0 * weightc<C>(k)) * cdot<C>(k, R.lid[0], R.lid[1], R.lid[2]) : own;
             };
             fin[a] = streamed(a, fs[b]);
             fin[b] = streamed(b, fs[a]);
@@ -1836,25 +1966,60 @@ __device__ __forceinline__ bool iface_one(const StepArgs& A, long long g) {
         rho = collide64_any(D.has_force, fin, [&](int a, double v) { dst[(unsigned)a * S + (unsigned)g] = v; }, R.omp,
                             R.omm, R.g);
     } else {
+        if constexpr (TWO) {
+            const float us = __fmaf_rn(ugz, ugz, __fmaf_rn(ugx, ugx, __fmul_rn(ugy, ugy)));
+            const float rg2 = __fmul_rn(3.f, __fmaf_rn(R.sigma2, kappa, pv));
+            const float wr1 = __fmul_rn(weightc<float>(1), rg2), wr2 = __fmul_rn(weightc<float>(7), rg2);
+            auto pair = [&](auto ac) {
+                constexpr int a = decltype(ac)::value;
+                const float cu = cdot32<a>(ugx, ugy, ugz), wr = a <= 6 ? wr1 : wr2;
+                const float inn = __fmaf_rn(-1.5f, us, __fmaf_rn(4.5f, __fmul_rn(cu, cu), 1.f)), c3 = __fmul_rn(3.f, cu);
+                auto one = [&](auto kc) {
+                    constexpr int k = decltype(kc)::value;
+                    constexpr char rg_ = two_kernel_rounding(k, sizeof(T) == 4, ONE, true);
+                    constexpr char rn_ = two_kernel_rounding(k, sizeof(T) == 4, ONE, false);
+                    const float own = fs[opp(k)];
+                    const uint8_t t = ty(k);
+                    const float gas = __fsub_rn(feq_both32<rg_>(wr, inn, c3), own);
+                    const float nrm = rg_ == rn_ ? gas : __fsub_rn(feq_both32<rn_>(wr, inn, c3), own);
+                    float v = t == GAS ? gas : fy[k];
+                    if (t < GAS && D.normal_rule && ((nmk >> k) & 1u)) v = nrm;
+                    if (t == OBS) {
+                        v = own;
+                        if (is_lid(k)) v = own + (6.f * weightc<float>(k)) * cdot<float>(k, R.lid[0], R.lid[1], R.lid[2]);
+                    }
+                    fin[k] = v;
+                };
+                one(std::integral_constant<int, a>{});
+                one(std::integral_constant<int, a + 1>{});
+            };
+            pair(std::integral_constant<int, 1>{}); pair(std::integral_constant<int, 3>{});
+            pair(std::integral_constant<int, 5>{}); pair(std::integral_constant<int, 7>{});
+            pair(std::integral_constant<int, 9>{}); pair(std::integral_constant<int, 11>{});
+            pair(std::integral_constant<int, 13>{}); pair(std::integral_constant<int, 15>{});
+            pair(std::integral_constant<int, 17>{});
+        } else {
 #pragma unroll
-        for (int a = 1; a < 19; ++a) {
-            const C fsb = fs[opp(a)];
-            const uint8_t tya = ty(a);
-            if (tya == OBS) {
-                fin[a] = fsb;
-            } else if (tya == LID) {
-                const C cuw = ((C)cx(a) * R.lid[0] + (C)cy(a) * R.lid[1]) + (C)cz(a) * R.lid[2];
-                fin[a] = fsb + ((C)6 * weightc<C>(a)) * cuw;
-            } else {
-                C fp, fm;
-                feq_pair<C>(a, rg, ugx, ugy, ugz, usg, fp, fm);
-                const C fga = (a & 1) ? fp + fm : fp - fm;
-                const C fgb = (a & 1) ? fp - fm : fp + fm;
-                if (tya == GAS) {
-                    fin[a] = (fga + fgb) - fsb;
+            for (int a = 1; a < 19; ++a) {
+                const C fsb = fs[opp(a)];
+                const uint8_t tya = ty(a);
+                if (tya == OBS) {
+                    fin[a] = fsb;
+                    if (is_lid(a)) {
+                        const C cuw = ((C)cx(a) * R.lid[0] + (C)cy(a) * R.lid[1]) + (C)cz(a) * R.lid[2];
+                        fin[a] = fsb + ((C)6 * weightc<C>(a)) * cuw;
+                    }
                 } else {
-                    fin[a] = fy[a];
-                    if (D.normal_rule && ((nmk >> a) & 1u)) fin[a] = (fga + fgb) - fsb;
+                    C fp, fm;
+                    feq_pair<C>(a, rg, ugx, ugy, ugz, usg, fp, fm);
+                    const C fga = (a & 1) ? fp + fm : fp - fm;
+                    const C fgb = (a & 1) ? fp - fm : fp + fm;
+                    if (tya == GAS) {
+                        fin[a] = (fga + fgb) - fsb;
+                    } else {
+                        fin[a] = fy[a];
+                        if (D.normal_rule && ((nmk >> a) & 1u)) fin[a] = (fga + fgb) - fsb;
+                    }
                 }
             }
         }
@@ -1876,7 +2041,17 @@ __device__ __forceinline__ bool iface_one(const StepArgs& A, long long g) {
     // the cell mass accumulates in FP64 for every form; fill / empty marks
     const double mnew = m0 + (double)dm;
     A.m[g] = mnew;
-    A.rhoi[g] = (double)rho;
+    ((C*)A.rhoi)[g] = rho;
+    IfOut<C> out{false, -1, 0};
+    if (A.fused) {
+        out.key = A.id[g];
+        C phn;
+        if constexpr (sizeof(C) == 8) phn = mnew / rho;
+        else phn = (float)mnew / rho;
+        ((C*)A.phi_next)[g] = phn;
+        ((C*)A.phit)[g] = clamp01(phn);
+        out.dv = volume_term_c(IFC, phn) - volume_term_c(IFC, phx);
+    }
     bool filled, emptied;
     if constexpr (sizeof(C) == 8) {
         filled = mnew > (1.0 + D.eps) * rho;
@@ -1893,8 +2068,9 @@ __device__ __forceinline__ bool iface_one(const StepArgs& A, long long g) {
         if (!has_gas) mk = MK_FILLED;
         else if (!has_liq) mk = MK_EMPTIED;
     }
-    A.mark[g] = mk;
-    return mk != MK_NONE;
+    out.marked = mk != MK_NONE;
+    if (out.marked) A.mark[g] = mk;   // (it is MK_NONE between steps)
+    return out;
 }
 
 // The interface cells of the list, one per thread, by a resident grid (block
@@ -1907,13 +2083,14 @@ __global__ void __launch_bounds__(IfThreads<T>::n, sizeof(T) == 8 ? 4 : 5) k_ifa
     const int cnt = *A.icount;
     for (long long base = (long long)blockIdx.x * IB; base < cnt; base += (long long)gridDim.x * IB) {
         const long long i = base + threadIdx.x;
-        bool mk = false;
+        IfOut<typename Form<T>::C> o{false, -1, 0};
         long long g = 0;
         if (i < cnt) {
             g = A.ilist[i];
-            mk = iface_one<T, ONE>(A, g);
+            o = iface_one<T, ONE, true>(A, g);
         }
-        list_append(A.mlist, A.mcount, mk, (int)g);
+        list_append(A.mlist, A.mcount, o.marked, (int)g);
+        if (A.fused) warp_add(A.vfx, o.dv != 0 ? o.key : -1, o.dv);
     }
 }
 
@@ -1963,13 +2140,14 @@ __global__ void __launch_bounds__(FSL_BLOCK, 2) k_stream_tile(StepArgs A) {
     const int ni = nil;
     for (int i0 = 0; i0 < ni; i0 += FSL_BLOCK) {
         const int i = i0 + threadIdx.x;
-        bool mk = false;
+        IfOut<typename Form<T>::C> o{false, -1, 0};
         long long g = 0;
         if (i < ni) {
             g = il[i];
-            mk = iface_one<T, ONE>(A, g);
+            o = iface_one<T, ONE, false>(A, g);
         }
-        list_append(A.mlist, A.mcount, mk, (int)g);
+        list_append(A.mlist, A.mcount, o.marked, (int)g);
+        if (A.fused) warp_add(A.vfx, o.dv != 0 ? o.key : -1, o.dv);
     }
 }
 
@@ -2193,7 +2371,7 @@ __device__ inline void convert_ab_phase(const StepArgs& A, int nm) {
                     A.id[z] = A.id[p];
                     bbox_extend(A.bbox, A.id[p], cz_.x, cz_.y, cz_.z);
                     A.m[z] = r;
-                    A.rhoi[z] = r;
+                    ((typename Form<T>::C*)A.rhoi)[z] = (typename Form<T>::C)r;
                     atomicAdd((unsigned long long*)&A.nif[d], 1ull);
                 }
             }
@@ -2257,29 +2435,8 @@ __device__ inline void convert_newgas_phase(const StepArgs& A) {
         for (int q = 0; q < 19; ++q)
             if (lane == q) Form<T>::st(f + (long long)q * S + z, q, fe[q]);
         if (lane == 19) A.m[z] = 0.0;
-        if (lane == 20) A.rhoi[z] = (double)rbar;
+        if (lane == 20) ((C*)A.rhoi)[z] = rbar;
     }
-}
-
-// Sum v over the lanes of the warp that share a key into base[key], one
-// atomic per distinct key (the values are fixed point, so the order of the
-// additions does not matter); key < 0 contributes nothing.  Every lane of the
-// warp must call.
-__device__ inline void warp_add(long long* base, int key, long long v) {
-    const unsigned full = 0xffffffffu;
-    const int k0 = __shfl_sync(full, key, 0);
-    if (__all_sync(full, key == k0)) {
-        if (k0 < 0) return;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(full, v, o);
-        if ((threadIdx.x & 31) == 0 && v != 0) atomicAdd((unsigned long long*)&base[k0], (unsigned long long)v);
-        return;
-    }
-    const unsigned peers = __match_any_sync(full, key);
-    long long sum = 0;
-    for (unsigned m = peers; m; m &= m - 1) sum += __shfl_sync(peers, v, __ffs(m) - 1);
-    if ((int)(threadIdx.x & 31) == __ffs(peers) - 1 && key >= 0 && sum != 0)
-        atomicAdd((unsigned long long*)&base[key], (unsigned long long)sum);
 }
 
 // 3x3x3 cube around a cell, bit k = (dx+1) + 3 (dy+1) + 9 (dz+1); bit 13 is the
@@ -2473,13 +2630,14 @@ __device__ inline void mark_affected(const StepArgs& A, const CclArgs& K, int d,
 
 // Unit normal n = -g / |g| of the fill level at cell w (Parker-Youngs gradient
 // g over the 3x3x3 stencil of the stencil fill levels), 0 where g = 0.
+template <typename C>
 __device__ inline void unit_normal_at(const StepArgs& A, const Dom& D, long long w, float& nx, float& ny, float& nz) {
     const Cell c = make_cell(D, w);
     float v[27];
 #pragma unroll
     for (int k = 0; k < 27; ++k) {
         const long long z = c.at(k % 3 - 1, (k / 3) % 3 - 1, k / 9 - 1);
-        v[k] = A.phitf ? A.phitf[z] : (float)A.phit[z];
+        v[k] = (float)((const C*)A.phit)[z];
     }
     float gx = 0.f, gy = 0.f, gz = 0.f;
 #pragma unroll
@@ -2502,13 +2660,14 @@ __device__ inline void unit_normal_at(const StepArgs& A, const Dom& D, long long
 // own bubble b (after this step's conversion) whose unit normals point in
 // opposite directions (n_i . n_j < -1/2): a liquid film between two parts of
 // one bubble, which may have cut it in two.
+template <typename C>
 __device__ inline bool antiparallel_normals(const StepArgs& A, const Dom& D, const Cell& c, long long g, int b) {
     float nxs[18], nys[18], nzs[18];
     int k = 0;
     for (int a = 1; a < 19; ++a) {
         const long long w = c.at(rcx(a), rcy(a), rcz(a));
         if (new_type(ctype(A.flag[w]), A.mark[w]) != IFC || A.id[w] != b) continue;
-        unit_normal_at(A, D, w, nxs[k], nys[k], nzs[k]);
+        unit_normal_at<C>(A, D, w, nxs[k], nys[k], nzs[k]);
         for (int j = 0; j < k; ++j)
             if (nxs[j] * nxs[k] + nys[j] * nys[k] + nzs[j] * nzs[k] < -0.5f) return true;
         ++k;
@@ -2522,6 +2681,7 @@ __device__ inline bool antiparallel_normals(const StepArgs& A, const Dom& D, con
 // triggers.  Taking the filled cells away one at a time in index order, each
 // removal must pass the local test with the lower-index filled cells already
 // gone and the higher-index ones still present, or the labelling runs.
+template <typename C>
 __device__ inline void convert_c_phase(const StepArgs& A, const CclArgs& K, int nm) {
     const int nl = *A.lcount;
     const int total = nm + nl;
@@ -2535,11 +2695,12 @@ __device__ inline void convert_c_phase(const StepArgs& A, const CclArgs& K, int 
         const uint8_t mk = A.mark[g];
         if (i < nm) {
             if (mk != MK_FILLED && mk != MK_EMPTIED) continue;   // emptied mark cancelled in phase A
-            const double mg = A.m[g], rg = A.rhoi[g];
+            const double mg = A.m[g], rg = (double)((const C*)A.rhoi)[g];
             // types and marks of the 26 neighbours, a plane of nine at a time:
             // rcv = interface after conversion, fgm = still gas / interface, or
             // filled in this step with a higher index
-            unsigned rcv = 0, fgm = 0;
+            // (old: interface before it as well)
+            unsigned rcv = 0, fgm = 0, old = 0;
 #pragma unroll
             for (int dz = -1; dz <= 1; ++dz) {
                 uint8_t fl[9], mz[9];
@@ -2556,6 +2717,7 @@ __device__ inline void convert_c_phase(const StepArgs& A, const CclArgs& K, int 
                     const uint8_t nt = new_type(fl[k], mz[k]);
                     const bool lf = fl[k] == IFC && (mz[k] == MK_FILLED || mz[k] == MK_CFILLED) && later[k];
                     rcv |= (unsigned)(nt == IFC) << (k + 9 * (dz + 1));
+                    old |= (unsigned)(fl[k] == IFC) << (k + 9 * (dz + 1));
                     fgm |= (unsigned)(nt == GAS || nt == IFC || lf) << (k + 9 * (dz + 1));
                 }
             }
@@ -2564,13 +2726,23 @@ __device__ inline void convert_c_phase(const StepArgs& A, const CclArgs& K, int 
             const int k = __popc(rcv);
             for (unsigned e = rcv; e; e &= e - 1) {
                 const int q = __ffs(e) - 1;
-                A.recv[c.at(q % 3 - 1, (q / 3) % 3 - 1, q / 9 - 1)] = step;   // pulls a share in phase D
+                const long long z = c.at(q % 3 - 1, (q / 3) % 3 - 1, q / 9 - 1);
+                // z pulls a share in phase D; a fused step lists the old interface cells among
+                // the receivers, once each (phase D finds the new ones in their own lists)
+                if (A.fused && ((old >> q) & 1u)) {
+                    if (atomicExch(&A.recv[z], step) != step) A.rlist[atomicAdd(A.rcount, 1)] = (int)z;
+                } else {
+                    A.recv[z] = step;
+                }
             }
             const double mex = (mk == MK_FILLED) ? mg - rg : mg;
             if (k > 0) A.exs[g] = mex / (double)k;
-            else atomicAdd((unsigned long long*)&A.pool[d], (unsigned long long)__double2ll_rn(mex * 1099511627776.0));
+            else {
+                atomicAdd((unsigned long long*)&A.pool[d], (unsigned long long)__double2ll_rn(mex * 1099511627776.0));
+                *A.pflag = 1;
+            }
             if (mk == MK_FILLED) {
-                const bool may_split = D.split_trigger ? antiparallel_normals(A, D, c, g, A.id[g])
+                const bool may_split = D.split_trigger ? antiparallel_normals<C>(A, D, c, g, A.id[g])
                                                        : !removal_is_local(fgm);
                 if (may_split) mark_affected(A, K, d, A.id[g]);   // its bubble may split
             }
@@ -2602,11 +2774,107 @@ __device__ inline void convert_c_phase(const StepArgs& A, const CclArgs& K, int 
     }
 }
 
-// Phase D, over the interface list and the two new-interface lists: receivers
-// pull the excess shares of converted neighbours in direction order and the
-// pool share, phi = m / rho (Eq. 9); converted cells take their new type;
-// bubble volumes change by exact fixed-point differences; the interface list
-// of the next step; reservoir drain; the graph condition of the labelling.
+// Reservoir drain of every domain whose seed cell is gas or interface after
+// this step's conversion, one thread per domain of block 0 (between the barriers
+// around phase C, where types and marks together name the new type).
+__device__ inline void reservoir_phase(const StepArgs& A) {
+    if (blockIdx.x != 0) return;
+    for (int d = threadIdx.x; d < A.ndom; d += blockDim.x) {
+        const Dom& D = get_dom(A, d);
+        if (D.seed < 0) continue;
+        const long long gs = D.off + D.seed;
+        const uint8_t nt = new_type(ctype(A.flag[gs]), A.mark[gs]);
+        const int b = A.id[gs];
+        if ((nt == GAS || nt == IFC) && b >= 0)
+            atomicAdd((unsigned long long*)&A.vxfx[b], (unsigned long long)(-D.rate_fx));
+    }
+}
+
+// What phase D changes outside the cell, summed per warp afterwards.
+struct DOut {
+    int key = -1, ckey = -1;       // bubble whose volume / cell count changes
+    long long dv = 0, dc = 0;
+    bool keep = false;             // still (or newly) an interface cell
+};
+
+// Phase D for one cell g of domain d: a converted cell takes its new type; any
+// other pulls the excess shares of converted neighbours in direction order and
+// the pool share, phi = m / rho (Eq. 9).  `ph0` is the fill level whose volume
+// term the bubble holds now.
+template <typename C>
+__device__ __forceinline__ DOut convert_d_cell(const StepArgs& A, long long g, int d, int step, const C* ph0) {
+    DOut o;
+    // everything the cell needs, loaded together
+    const uint8_t f = A.flag[g];
+    const uint8_t mk = A.mark[g];
+    o.key = A.id[g];
+    const double m0 = A.m[g];
+    const C rh = ((const C*)A.rhoi)[g], p0 = ph0[g];
+    const int rs = A.recv[g];
+    const long long nI = A.nif[d];
+    const long long pool = A.pool[d];
+    const uint8_t t = ctype(f);
+    C* phit = (C*)A.phit;
+    if (t == IFC && mk == MK_CFILLED) {
+        o.dv = -volume_term_c(IFC, p0);
+        o.ckey = o.key;
+        o.dc = -1;
+        A.flag[g] = (uint8_t)((f & ~K_TYPE) | LIQ);
+        phit[g] = (C)1;
+        A.id[g] = -1;
+        A.mark[g] = MK_NONE;
+        return o;
+    }
+    if (t == IFC && mk == MK_CEMPTIED) {
+        o.dv = FSL_VOL_ONE - volume_term_c(IFC, p0);
+        A.flag[g] = (uint8_t)((f & ~K_TYPE) | GAS);
+        phit[g] = (C)0;
+        A.m[g] = 0.0;
+        A.mark[g] = MK_NONE;
+        return o;
+    }
+    double sm = m0;
+    if (rs == step) {
+        // a converted neighbour named this cell among its receivers: all
+        // eighteen step stamps first, then the shares of the converted ones,
+        // added in direction order
+        const Dom& D = get_dom(A, d);
+        const Cell c = make_cell(D, g);
+        int cs[19];
+#pragma unroll
+        for (int a = 1; a < 19; ++a) cs[a] = A.cstep[c.at(cx(a), cy(a), cz(a))];
+        double ex[19];
+#pragma unroll
+        for (int a = 1; a < 19; ++a) ex[a] = cs[a] == step ? A.exs[c.at(cx(a), cy(a), cz(a))] : 0.0;
+#pragma unroll
+        for (int a = 1; a < 19; ++a)
+            if (cs[a] == step) sm = sm + ex[a];
+    }
+    if (nI > 0 && pool != 0) {
+        const double share = ((double)pool * 9.094947017729282379150390625e-13) / (double)nI;
+        sm = sm + share;
+    }
+    A.m[g] = sm;
+    C phn;
+    if constexpr (sizeof(C) == 8) phn = sm / rh;
+    else phn = (float)sm / rh;   // the conversion is the cell's only FP64-pipe work
+    ((C*)A.phi_next)[g] = phn;
+    phit[g] = clamp01(phn);
+    o.dv = volume_term_c(IFC, phn) - volume_term_c(t, p0);
+    if (t != IFC) {
+        A.flag[g] = (uint8_t)((f & ~K_TYPE) | IFC);
+        A.mark[g] = MK_NONE;
+    }
+    if (t == LIQ) { o.ckey = o.key; o.dc = 1; }
+    o.keep = true;
+    return o;
+}
+
+// Phase D, over the interface list and the two new-interface lists: bubble
+// volumes change by exact fixed-point differences; the interface list of the
+// next step.  Used after the stream-collide forms whose interface kernel does
+// not form the fill levels.
+template <typename C>
 __device__ inline void convert_d_phase(const StepArgs& A) {
     const int ni = *A.icount, ng = *A.gcount, nl = *A.lcount;
     const int total = ni + ng + nl;
@@ -2619,90 +2887,13 @@ __device__ inline void convert_d_phase(const StepArgs& A) {
         long long g = 0;
         if (valid) g = i < ni ? A.ilist[i] : (i < ni + ng ? A.glist[i - ni] : A.llist[i - ni - ng]);
         const int d = valid ? block_dom(A, g) : 0;
-        int key = -1;
-        long long dv = 0;
-        int ckey = -1;
-        long long dc = 0;
-        bool keep = false;
-        if (valid) {
-            // everything the cell needs, loaded together
-            const uint8_t f = A.flag[g];
-            const uint8_t mk = A.mark[g];
-            key = A.id[g];
-            const double m0 = A.m[g], rh = A.rhoi[g];
-            // FP32-collide forms: fill levels and volume terms from the FP32 copies,
-            // which are the only ones kept (the FP64 fill level and stencil level
-            // belong to the FP64 form)
-            const bool f32 = A.phif != nullptr;
-            const double ph0 = f32 ? 0.0 : A.phi[g];
-            const float ph0f = f32 ? A.phif[g] : 0.f;
-            const int rs = A.recv[g];
-            const long long nI = A.nif[d];
-            const long long pool = A.pool[d];
-            const uint8_t t = ctype(f);
-            if (t == IFC && mk == MK_CFILLED) {
-                dv = f32 ? -volume_term_f(IFC, ph0f) : -volume_term(IFC, ph0);
-                ckey = key;
-                dc = -1;
-                A.flag[g] = (uint8_t)((f & ~K_TYPE) | LIQ);
-                if (f32) { A.phif[g] = 1.f; A.phitf[g] = 1.f; }
-                else { A.phi[g] = 1.0; A.phit[g] = 1.0; }
-                A.id[g] = -1;
-                A.mark[g] = MK_NONE;
-            } else if (t == IFC && mk == MK_CEMPTIED) {
-                dv = FSL_VOL_ONE - (f32 ? volume_term_f(IFC, ph0f) : volume_term(IFC, ph0));
-                A.flag[g] = (uint8_t)((f & ~K_TYPE) | GAS);
-                if (f32) { A.phif[g] = 0.f; A.phitf[g] = 0.f; }
-                else { A.phi[g] = 0.0; A.phit[g] = 0.0; }
-                A.m[g] = 0.0;
-                A.mark[g] = MK_NONE;
-            } else {
-                double sm = m0;
-                if (rs == step) {
-                    // a converted neighbour listed this cell among its receivers:
-                    // all eighteen step stamps first, then the shares of the
-                    // converted ones, added in direction order
-                    const Dom& D = get_dom(A, d);
-                    const Cell c = make_cell(D, g);
-                    int cs[19];
-#pragma unroll
-                    for (int a = 1; a < 19; ++a) cs[a] = A.cstep[c.at(cx(a), cy(a), cz(a))];
-                    double ex[19];
-#pragma unroll
-                    for (int a = 1; a < 19; ++a) ex[a] = cs[a] == step ? A.exs[c.at(cx(a), cy(a), cz(a))] : 0.0;
-#pragma unroll
-                    for (int a = 1; a < 19; ++a)
-                        if (cs[a] == step) sm = sm + ex[a];
-                }
-                if (nI > 0 && pool != 0) {
-                    const double share = ((double)pool * 9.094947017729282379150390625e-13) / (double)nI;
-                    sm = sm + share;
-                }
-                A.m[g] = sm;
-                if (f32) {
-                    // phi = m / rho in FP32 (Eq. 9); three conversions are the
-                    // only FP64-pipe work of the cell
-                    const float phf = (float)sm / (float)rh;
-                    A.phif[g] = phf;
-                    A.phitf[g] = fminf(fmaxf(phf, 0.f), 1.f);
-                    dv = volume_term_f(IFC, phf) - volume_term_f(t, ph0f);
-                } else {
-                    const double phn = sm / rh;
-                    const long long told = volume_term(t, ph0);
-                    A.phi[g] = phn;
-                    A.phit[g] = phn < 0.0 ? 0.0 : (phn > 1.0 ? 1.0 : phn);
-                    dv = volume_term(IFC, phn) - told;
-                }
-                if (t != IFC) A.flag[g] = (uint8_t)((f & ~K_TYPE) | IFC);
-                if (t == LIQ) { ckey = key; dc = 1; }
-                keep = true;
-            }
-        }
-        warp_add(A.vfx, dv != 0 ? key : -1, dv);
-        warp_add(A.ncells, ckey, dc);
-        if (A.ndom == 1) kept += keep ? 1 : 0;
-        else warp_add(A.icnt, keep ? d : -1, 1);
-        if (!A.order) list_append(A.ilist_next, A.icount_next, keep, (int)g);
+        DOut o;
+        if (valid) o = convert_d_cell<C>(A, g, d, step, (const C*)A.phi);
+        warp_add(A.vfx, o.dv != 0 ? o.key : -1, o.dv);
+        warp_add(A.ncells, o.ckey, o.dc);
+        if (A.ndom == 1) kept += o.keep ? 1 : 0;
+        else warp_add(A.icnt, o.keep ? d : -1, 1);
+        if (!A.order) list_append(A.ilist_next, A.icount_next, o.keep, (int)g);
     }
     if (A.ndom == 1) {
         // one domain: the interface count by one atomic per warp
@@ -2710,24 +2901,69 @@ __device__ inline void convert_d_phase(const StepArgs& A) {
         for (int o = 16; o > 0; o >>= 1) kept += __shfl_down_sync(0xffffffffu, kept, o);
         if ((threadIdx.x & 31) == 0 && kept) atomicAdd((unsigned long long*)&A.icnt[0], (unsigned long long)kept);
     }
-    if (blockIdx.x == 0) {
-        // reservoir drain of every domain whose seed cell is still gas or
-        // interface (types read through the marks, which stay consistent
-        // while other threads update the flags), one thread per domain
-        for (int d = threadIdx.x; d < A.ndom; d += blockDim.x) {
-            const Dom& D = get_dom(A, d);
-            if (D.seed < 0) continue;
-            const long long gs = D.off + D.seed;
-            const uint8_t nt = new_type(ctype(A.flag[gs]), A.mark[gs]);
-            const int b = A.id[gs];
-            if ((nt == GAS || nt == IFC) && b >= 0)
-                atomicAdd((unsigned long long*)&A.vxfx[b], (unsigned long long)(-D.rate_fx));
+}
+
+__device__ inline unsigned ifc_mask16(const uint8_t* flag, long long j);
+
+// Fused step with pooled excess mass (rare: a converted cell without any
+// interface neighbour): the interface cells that neither converted nor receive
+// a share take the pool share here, found by their types and marks, which no
+// thread changes before the barrier that follows.
+template <typename C>
+__device__ inline void convert_pool_phase(const StepArgs& A) {
+    const int step = *A.stepno;
+    const long long words = A.stride / 16, stride = (long long)gridDim.x * blockDim.x;
+    for (long long base = (long long)blockIdx.x * blockDim.x; base < words; base += stride) {
+        const long long j = base + threadIdx.x;
+        const int d = j < words ? block_dom(A, 16 * j) : 0;
+        unsigned m = j < words && A.pool[d] != 0 && A.nif[d] > 0 ? ifc_mask16(A.flag, j) : 0u;
+        while (__any_sync(0xffffffffu, m != 0)) {
+            const long long g = 16 * j + (m ? __ffs(m) - 1 : 0);
+            DOut o;
+            if (m) {
+                const uint8_t mk = A.mark[g];
+                if (mk != MK_CFILLED && mk != MK_CEMPTIED && A.recv[g] != step)
+                    o = convert_d_cell<C>(A, g, d, step, (const C*)A.phi_next);
+            }
+            warp_add(A.vfx, o.dv != 0 ? o.key : -1, o.dv);
+            m &= m - 1;
         }
-        if (threadIdx.x == 0) *A.mcount = 0;
     }
 }
 
-
+// Phase D of a fused step: the marked cells that converted, the receivers of
+// excess mass, and the new interface cells.  The interface count follows from
+// the conversions (nif).
+template <typename C>
+__device__ inline void convert_d_fused(const StepArgs& A, int nm) {
+    if (blockIdx.x == 0)
+        for (int d = threadIdx.x; d < A.ndom; d += blockDim.x) A.icnt[d] = A.nif[d];
+    if (nm == 0) return;
+    const int nr = *A.rcount, ng = *A.gcount, nl = *A.lcount;
+    const int total = nm + nr + ng + nl;
+    const int step = *A.stepno;
+    const int stride = gridDim.x * blockDim.x;
+    for (int base = blockIdx.x * blockDim.x; base < total; base += stride) {
+        const int i = base + threadIdx.x;
+        long long g = -1;
+        if (i < nm) {
+            g = A.mlist[i];
+            // converted in this step (an emptied mark that phase A cancelled is
+            // an ordinary interface cell, listed if it receives)
+            if (A.cstep[g] != step) g = -1;
+        } else if (i < nm + nr) {
+            g = A.rlist[i - nm];
+        } else if (i < nm + nr + ng) {
+            g = A.glist[i - nm - nr];
+        } else if (i < total) {
+            g = A.llist[i - nm - nr - ng];
+        }
+        DOut o;
+        if (g >= 0) o = convert_d_cell<C>(A, g, block_dom(A, g), step, (const C*)A.phi_next);
+        warp_add(A.vfx, o.dv != 0 ? o.key : -1, o.dv);
+        warp_add(A.ncells, o.ckey, o.dc);
+    }
+}
 
 // --------------------------------------------- connected-component labelling
 // Bubbles are the 18-connected components of gas + interface cells (Sec. 2.3);
@@ -2989,6 +3225,7 @@ __device__ inline void hash_add(const CclArgs& K, unsigned long long key, long l
 
 // Phase 4: new volumes and cell counts per component, overlap volumes V_{c,b}
 // of new component c with old bubble b, new slots into the id field.
+template <typename C>
 __device__ inline void ccl_pairs_phase(const StepArgs& A, const CclArgs& K) {
     const int np = *K.np;
     FSL_LIST_LOOP(i, np) {
@@ -3003,7 +3240,8 @@ __device__ inline void ccl_pairs_phase(const StepArgs& A, const CclArgs& K) {
             const int r = K.lab[g];
             c = (r >= 0 && K.lab[r] == r) ? K.aux[r] : -1;
             const uint8_t ty = ctype(A.flag[g]);
-            term = A.phif ? volume_term_f(ty, A.phif[g]) : volume_term(ty, A.phi[g]);
+            // (the initial pass runs before any step)
+            term = volume_term_c(ty, K.initial ? ((const C*)A.phi)[g] : ((const C*)A.phi_next)[g]);
         }
         warp_add(K.nvfx, c, term);
         warp_add(K.nncells, c, c >= 0 ? 1 : 0);
@@ -3148,22 +3386,44 @@ __global__ void __launch_bounds__(FSL_CONV_THREADS, 3) k_convert(StepArgs A, Ccl
     // no cell filled or emptied (the usual step of a quiet lattice): phases A to
     // C have nothing to do, and phase D needs no barrier before it (5 us of the
     // kernel's 10 us on a 32^3 lattice)
+    using C = typename Form<T>::C;
     const int nm = *A.mcount;
     bool relabel = false;
     if (nm > 0 || A.bar_extra) {
         convert_ab_phase<T>(A, nm);
         if (!grid_barrier(A)) return;
-        convert_c_phase(A, K, nm);
+        reservoir_phase(A);
+        convert_c_phase<C>(A, K, nm);
         convert_newgas_phase<T>(A);
         if (!grid_barrier(A)) return;
         relabel = *(volatile int*)A.trig != 0;   // final after phase C
+    } else {
+        reservoir_phase(A);
     }
-    convert_d_phase(A);
+    if (A.fused) {
+        if (*(volatile int*)A.pflag != 0) {
+            convert_pool_phase<C>(A);
+            if (!grid_barrier(A)) return;
+        }
+        convert_d_fused<C>(A, nm);
+    } else {
+        convert_d_phase<C>(A);
+    }
+    // (every block has read mcount: with marked cells there were barriers since)
+    if (blockIdx.x == 0 && threadIdx.x == 0) *A.mcount = 0;
     if (A.order) {
-        if (!grid_barrier(A)) return;
-        order_count_phase(A);
-        if (!grid_barrier(A)) return;
-        order_write_phase(A);
+        if (nm > 0) {
+            if (!grid_barrier(A)) return;
+            order_count_phase(A);
+            if (!grid_barrier(A)) return;
+            order_write_phase(A);
+        } else {
+            // nothing converted: the list stays as it is
+            const int ni = *A.icount;
+            for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ni; i += gridDim.x * blockDim.x)
+                A.ilist_next[i] = A.ilist[i];
+            if (blockIdx.x == 0 && threadIdx.x == 0) *A.icount_next = ni;
+        }
     }
     if (!relabel) return;
     if (!grid_barrier(A)) return;
@@ -3175,11 +3435,20 @@ __global__ void __launch_bounds__(FSL_CONV_THREADS, 3) k_convert(StepArgs A, Ccl
     if (!grid_barrier(A)) return;
     ccl_compress_phase(A, K);
     if (!grid_barrier(A)) return;
-    ccl_pairs_phase(A, K);
+    ccl_pairs_phase<C>(A, K);
     if (!grid_barrier(A)) return;
     ccl_table_phase(A, K);
     if (!grid_barrier(A)) return;
     ccl_install_phase(A, K);
+}
+
+// The interface list of the present state in cell order (into ilist_next), by
+// the same two passes, as a cooperative launch of its own.
+template <typename T>
+__global__ void __launch_bounds__(FSL_CONV_THREADS) k_order(StepArgs A) {
+    order_count_phase(A);
+    if (!grid_barrier(A)) return;
+    order_write_phase(A);
 }
 
 // Initial state: validate the closed interface layer, f = f_eq(rho, u),
@@ -3209,20 +3478,18 @@ __global__ void __launch_bounds__(FSL_BLOCK) k_init_state(StepArgs A, int d, con
     A.id[g] = -1;
     A.exs[g] = 0.0;
     double ph = (t == LIQ) ? 1.0 : (t == IFC ? fill[l] : 0.0);
-    A.phi[g] = ph;
-    const double pht = (t == LIQ || t == OBS || t == LID) ? 1.0 : (t == GAS ? 0.0 : (ph < 0.0 ? 0.0 : (ph > 1.0 ? 1.0 : ph)));
-    A.phit[g] = pht;
-    if (A.phif) { A.phif[g] = (float)ph; A.phitf[g] = (float)pht; }
+    ((C*)A.phi_next)[g] = (C)ph;
+    ((C*)A.phit)[g] = (C)((t == LIQ || t == OBS || t == LID) ? 1.0 : (t == GAS ? 0.0 : clamp01(ph)));
     T* f = (T*)A.fdst;
     if (t == LIQ || t == IFC) {
         C fe[19];
         feq_all<C>((C)rho[l], (C)u[l], (C)u[D.n + l], (C)u[2 * (long long)D.n + l], fe);
         for (int a = 0; a < 19; ++a) Form<T>::st(f + (long long)a * S + g, a, fe[a]);
-        A.rhoi[g] = rho[l];
+        ((C*)A.rhoi)[g] = (C)rho[l];
         A.m[g] = (t == IFC) ? fill[l] * rho[l] : rho[l];
     } else {
         for (int a = 0; a < 19; ++a) Form<T>::st(f + (long long)a * S + g, a, (C)weight(a));
-        A.rhoi[g] = 0.0;
+        ((C*)A.rhoi)[g] = (C)0;
         A.m[g] = 0.0;
     }
 }
@@ -3396,6 +3663,7 @@ template <typename T> int stream_blocks_per_sm(int form, bool one);
 template <typename T> cudaError_t launch_convert(const StepArgs& A, const CclArgs& K, int nblocks, cudaStream_t s,
                                                  bool pdl);
 template <typename T> int convert_blocks_per_sm();
+template <typename T> cudaError_t launch_order(const StepArgs& A, int nblocks, cudaStream_t s);
 template <typename T> void launch_init_state(const StepArgs& A, int d, int n, const uint8_t* fl, const double* fill,
                                              const double* rho, const double* u, cudaStream_t s);
 template <typename T> void launch_export_pdf(const void* f, long long S, long long off, int n, double* pdf,
@@ -3516,6 +3784,18 @@ template <typename T> void launch_mass_partials(const void* f, const uint8_t* fl
         cfg.attrs = at;                                                                                      \
         cfg.numAttrs = pdl ? 2 : 1;   /* after a join of two streams: a plain dependency */               \
         return cudaLaunchKernelEx(&cfg, k_convert<T>, A, K);                                                 \
+    }                                                                                                        \
+    template <> cudaError_t launch_order<T>(const StepArgs& A, int nb, cudaStream_t s) {                     \
+        cudaLaunchConfig_t cfg = {};                                                                         \
+        cfg.gridDim = dim3((unsigned)nb);                                                                    \
+        cfg.blockDim = dim3(FSL_CONV_THREADS);                                                               \
+        cfg.stream = s;                                                                                      \
+        cudaLaunchAttribute at[1];                                                                           \
+        at[0].id = cudaLaunchAttributeCooperative;                                                           \
+        at[0].val.cooperative = 1;                                                                           \
+        cfg.attrs = at;                                                                                      \
+        cfg.numAttrs = 1;                                                                                    \
+        return cudaLaunchKernelEx(&cfg, k_order<T>, A);                                                      \
     }                                                                                                        \
     template <> int convert_blocks_per_sm<T>() {                                                             \
         int nb = 0;                                                                                          \
