@@ -844,6 +844,18 @@ __device__ inline Pull make_pull(const Dom& D, long long g) {
     return p;
 }
 
+// PDF of direction a at a cell: the plane's base is the same for every thread (a
+// uniform 64-bit sum) and the cell a 32-bit byte offset (19 planes of 8 B stay
+// addressable: at most 226 M cells), so an access costs one 32-bit operation for
+// its address, or none where the cell is the thread's own, instead of a 64-bit
+// multiply-add per plane.
+template <typename T> __device__ __forceinline__ const T* pdf_at(const T* f, long long S, int a, unsigned cell) {
+    return (const T*)((const char*)(f + a * S) + (size_t)(cell * (unsigned)sizeof(T)));
+}
+template <typename T> __device__ __forceinline__ T* pdf_at(T* f, long long S, int a, unsigned cell) {
+    return (T*)((char*)(f + a * S) + (size_t)(cell * (unsigned)sizeof(T)));
+}
+
 // Liquid cells: stream with half-way bounce-back (Eq. 7) and collide (Eq. 6) for
 // liquid cells.  Only cells flagged as touching a wall read the types of
 // their neighbours; a liquid cell never touches gas (closed interface layer).
@@ -860,11 +872,12 @@ __device__ __forceinline__ void liquid_one(const StepArgs& A, long long g, uint8
     if constexpr (Form<T>::shifted) {
         // deviations from w_a all the way through
         float d[19];
-        d[0] = Form<T>::ld_dev(src + gi);
+        d[0] = Form<T>::ld_dev(pdf_at(src, S, 0, gi));
         if (!(f & K_WALL)) {
 #pragma unroll
             for (int a = 1; a < 19; ++a)
-                d[a] = Form<T>::ld_dev(src + a * S + (unsigned)(gi + P.ox[1 - cx(a)] + P.oy[1 - cy(a)] + P.oz[1 - cz(a)]));
+                d[a] = Form<T>::ld_dev(
+                    pdf_at(src, S, a, (unsigned)(gi + P.ox[1 - cx(a)] + P.oy[1 - cy(a)] + P.oz[1 - cz(a)])));
         } else {
             // all neighbour types first, then every load with its address
             // chosen without a branch (two memory latencies, not eighteen)
@@ -873,7 +886,8 @@ __device__ __forceinline__ void liquid_one(const StepArgs& A, long long g, uint8
                 const unsigned y = (unsigned)(gi + P.ox[1 - cx(a)] + P.oy[1 - cy(a)] + P.oz[1 - cz(a)]);
                 const uint8_t t = ctype(A.flag[y]);
                 // bounce-back reads the cell's own opposite PDF (w_a = w_abar)
-                const float v = Form<T>::ld_dev(src + ((t == OBS || t == LID) ? opp(a) * S + gi : a * S + y));
+                const bool bb = t == OBS || t == LID;
+                const float v = Form<T>::ld_dev(bb ? pdf_at(src, S, opp(a), gi) : pdf_at(src, S, a, y));
                 d[a] = t == LID ? v + (6.f * weightc<float>(a)) * cdot<float>(a, R.lid[0], R.lid[1], R.lid[2]) : v;
             }
         }
@@ -884,14 +898,15 @@ __device__ __forceinline__ void liquid_one(const StepArgs& A, long long g, uint8
             collide_dev<false>(d, dout, R.omp, R.omm, 0.f, 0.f, 0.f);
         if (!(dout[0] == dout[0])) set_status(A.status, ST_NAN);
 #pragma unroll
-        for (int a = 0; a < 19; ++a) Form<T>::st_dev(dst + a * S + gi, dout[a]);
+        for (int a = 0; a < 19; ++a) Form<T>::st_dev(pdf_at(dst, S, a, gi), dout[a]);
     } else {
         C fin[19];
-        fin[0] = Form<T>::ld(src + gi, 0);
+        fin[0] = Form<T>::ld(pdf_at(src, S, 0, gi), 0);
         if (!(f & K_WALL)) {
 #pragma unroll
             for (int a = 1; a < 19; ++a)
-                fin[a] = Form<T>::ld(src + a * S + (unsigned)(gi + P.ox[1 - cx(a)] + P.oy[1 - cy(a)] + P.oz[1 - cz(a)]), a);
+                fin[a] = Form<T>::ld(
+                    pdf_at(src, S, a, (unsigned)(gi + P.ox[1 - cx(a)] + P.oy[1 - cy(a)] + P.oz[1 - cz(a)])), a);
         } else {
             unsigned bm = 0, lm = 0;   // links from an obstacle / the lid
 #pragma unroll
@@ -904,7 +919,7 @@ __device__ __forceinline__ void liquid_one(const StepArgs& A, long long g, uint8
             for (int a = 1; a < 19; ++a) {
                 const unsigned y = (unsigned)(gi + P.ox[1 - cx(a)] + P.oy[1 - cy(a)] + P.oz[1 - cz(a)]);
                 // w_a = w_abar, so the stored form of direction abar reads the same
-                fin[a] = Form<T>::ld(src + (((bm >> a) & 1u) ? opp(a) * S + gi : a * S + y), a);
+                fin[a] = Form<T>::ld(((bm >> a) & 1u) ? pdf_at(src, S, opp(a), gi) : pdf_at(src, S, a, y), a);
             }
             if (lm) {
 #pragma unroll
@@ -914,12 +929,13 @@ __device__ __forceinline__ void liquid_one(const StepArgs& A, long long g, uint8
         }
         C rho;
         if constexpr (sizeof(C) == 8) {
-            rho = collide64_any(D.has_force, fin, [&](int a, double v) { dst[a * S + gi] = v; }, R.omp, R.omm, R.g);
+            rho = collide64_any(D.has_force, fin, [&](int a, double v) { *pdf_at(dst, S, a, gi) = (T)v; }, R.omp,
+                                R.omm, R.g);
         } else {
             C fout[19];
             rho = collide_any<C>(D.has_force, fin, fout, R.omp, R.omm, R.g[0], R.g[1], R.g[2]);
 #pragma unroll
-            for (int a = 0; a < 19; ++a) Form<T>::st(dst + a * S + gi, a, fout[a]);
+            for (int a = 0; a < 19; ++a) Form<T>::st(pdf_at(dst, S, a, gi), a, fout[a]);
         }
         if (!(rho == rho)) set_status(A.status, ST_NAN);
     }
@@ -952,41 +968,47 @@ __device__ __forceinline__ void liquid_pairs(const StepArgs& A, long long bid) {
     if (!v0 && !v1) return;
     const Dom& D = dom_at<ONE>(A, g0);
     const Par<float> R = par_of<float>(D);
-    const unsigned S = (unsigned)A.stride, gi = (unsigned)g0;
+    const long long S = A.stride;
+    const unsigned gi = (unsigned)g0;
     const T* __restrict__ src = (const T*)A.fsrc;
     T* __restrict__ dst = (T*)A.fdst;
     float2 d[19];
-    if (!((f0 | f1) & K_WALL) && !(D.nx & 1)) {
-        // even nx: x0 is even and both cells lie in one row, so the y / z
-        // offsets of a link are common to the pair and only its x offsets
-        // differ: cell 0 pulls x - 1 from the row's end when x0 = 0, cell 1
-        // pulls x + 1 from the row's start when x0 + 1 = nx - 1.  Links along
-        // x = const read both sources with one aligned 32-bit load.
-        int x, y, z;
-        local_xyz(D, (int)(g0 - D.off), x, y, z);
+    int x, y, z;
+    local_xyz(D, (int)(g0 - D.off), x, y, z);
+    if (!((f0 | f1) & K_WALL) && x + 1 < D.nx) {
+        // both cells lie in one row, so the y / z offsets of a link are common
+        // to the pair and only its x offsets differ: cell 0 pulls x - 1 from the
+        // row's end when x0 = 0, cell 1 pulls x + 1 from the row's start when
+        // x0 + 1 = nx - 1.  With an even nx (x0 is then even) links along x =
+        // const read both sources with one aligned 32-bit load.
         const int sy = D.nx, sz = D.nx * D.ny;
         const int oy[3] = {y == 0 ? (D.ny - 1) * sy : -sy, 0, y == D.ny - 1 ? -(D.ny - 1) * sy : sy};
         const int oz[3] = {z == 0 ? (D.nz - 1) * sz : -sz, 0, z == D.nz - 1 ? -(D.nz - 1) * sz : sz};
         const int xm0 = x == 0 ? D.nx - 1 : -1;                 // cell 0, source x - 1
         const int xp1 = x + 2 == D.nx ? 2 - D.nx : 2;           // cell 1, source x + 1 (from cell 0)
+        auto pull = [&](auto even) {
 #pragma unroll
-        for (int a = 0; a < 19; ++a) {
-            const unsigned r = gi + (unsigned)(oy[1 - cy(a)] + oz[1 - cz(a)]);
-            if (cx(a) == 0) {
-                d[a] = Form<T>::ld_dev2(src + (a * S + r));
-            } else if (cx(a) > 0) {   // sources x - 1: cell 0's per x0, cell 1's is cell 0's column
-                d[a] = make_float2(Form<T>::ld_dev(src + (a * S + r + (unsigned)xm0)), Form<T>::ld_dev(src + (a * S + r)));
-            } else {                  // sources x + 1: cell 0's is cell 1's column
-                d[a] = make_float2(Form<T>::ld_dev(src + (a * S + r + 1u)), Form<T>::ld_dev(src + (a * S + r + (unsigned)xp1)));
+            for (int a = 0; a < 19; ++a) {
+                const unsigned r = gi + (unsigned)(oy[1 - cy(a)] + oz[1 - cz(a)]);
+                auto ld = [&](unsigned cell) { return Form<T>::ld_dev(pdf_at(src, S, a, cell)); };
+                if (cx(a) == 0) {
+                    if constexpr (decltype(even)::value) d[a] = Form<T>::ld_dev2(pdf_at(src, S, a, r));
+                    else d[a] = make_float2(ld(r), ld(r + 1u));
+                } else if (cx(a) > 0) {   // sources x - 1: cell 0's per x0, cell 1's is cell 0's column
+                    d[a] = make_float2(ld(r + (unsigned)xm0), ld(r));
+                } else {                  // sources x + 1: cell 0's is cell 1's column
+                    d[a] = make_float2(ld(r + 1u), ld(r + (unsigned)xp1));
+                }
             }
-        }
+        };
+        if (!(D.nx & 1)) pull(std::true_type{});
+        else pull(std::false_type{});
     } else {
         const Pull P0 = make_pull(D, g0), P1 = make_pull(D, g0 + 1);
-        // walls, or odd nx (the pair may straddle two rows): every link of
-        // each cell on its own, a wall cell's bounced links chosen without a
-        // branch
+        // walls, or a pair that straddles two rows: every link of each cell on
+        // its own, a wall cell's bounced links chosen without a branch
         const bool k0 = v0 && (f0 & K_WALL), k1 = v1 && (f1 & K_WALL);
-        d[0] = make_float2(Form<T>::ld_dev(src + gi), Form<T>::ld_dev(src + gi + 1u));
+        d[0] = make_float2(Form<T>::ld_dev(pdf_at(src, S, 0, gi)), Form<T>::ld_dev(pdf_at(src, S, 0, gi + 1u)));
 #pragma unroll
         for (int a = 1; a < 19; ++a) {
             const unsigned y0 = gi + (unsigned)(P0.ox[1 - cx(a)] + P0.oy[1 - cy(a)] + P0.oz[1 - cz(a)]);
@@ -994,8 +1016,9 @@ __device__ __forceinline__ void liquid_pairs(const StepArgs& A, long long bid) {
             const uint8_t t0 = k0 ? ctype(A.flag[y0]) : (uint8_t)LIQ;
             const uint8_t t1 = k1 ? ctype(A.flag[y1]) : (uint8_t)LIQ;
             // bounce-back reads the cell's own opposite PDF (w_a = w_abar)
-            float x0 = Form<T>::ld_dev(src + ((t0 == OBS || t0 == LID) ? opp(a) * S + gi : a * S + y0));
-            float x1 = Form<T>::ld_dev(src + ((t1 == OBS || t1 == LID) ? opp(a) * S + gi + 1u : a * S + y1));
+            const bool b0 = t0 == OBS || t0 == LID, b1 = t1 == OBS || t1 == LID;
+            float x0 = Form<T>::ld_dev(b0 ? pdf_at(src, S, opp(a), gi) : pdf_at(src, S, a, y0));
+            float x1 = Form<T>::ld_dev(b1 ? pdf_at(src, S, opp(a), gi + 1u) : pdf_at(src, S, a, y1));
             const float lidt = (6.f * weightc<float>(a)) * cdot<float>(a, R.lid[0], R.lid[1], R.lid[2]);
             if (t0 == LID) x0 += lidt;
             if (t1 == LID) x1 += lidt;
@@ -1009,7 +1032,7 @@ __device__ __forceinline__ void liquid_pairs(const StepArgs& A, long long bid) {
     const bool both = v0 && v1;
     auto out = [&](int a, float2 v) {
         if (a == 0 && ((v0 && !(v.x == v.x)) || (v1 && !(v.y == v.y)))) set_status(A.status, ST_NAN);
-        Form<T>::st_dev2m(dst + (a * S + gi), v, both, v0 && !v1, v1 && !v0);
+        Form<T>::st_dev2m(pdf_at(dst, S, a, gi), v, both, v0 && !v1, v1 && !v0);
     };
     if (D.has_force)
         collide_dev2<true>(d, out, R.omp, R.omm, R.g[0], R.g[1], R.g[2]);
@@ -1865,7 +1888,7 @@ __device__ __forceinline__ IfOut<typename Form<T>::C> iface_one(const StepArgs& 
     using C = typename Form<T>::C;
     const Dom& D = dom_at<ONE>(A, g);
     const Par<C> R = par_of<C>(D);
-    const unsigned S = (unsigned)A.stride;
+    const long long S = A.stride;
     const T* __restrict__ src = (const T*)A.fsrc;
     T* __restrict__ dst = (T*)A.fdst;
     const C* __restrict__ phic = (const C*)A.phi;
@@ -1883,14 +1906,14 @@ __device__ __forceinline__ IfOut<typename Form<T>::C> iface_one(const StepArgs& 
     // and the fill level, where the link has a use for them: a gas or wall source
     // streams nothing in, and only interface neighbours weigh the mass exchange
     C fs[19], fy[19], phy[19];
-    fs[0] = Form<T>::ld(src + (unsigned)g, 0);
+    fs[0] = Form<T>::ld(pdf_at(src, S, 0, (unsigned)g), 0);
 #pragma unroll
     for (int a = 1; a < 19; ++a) {
-        fs[a] = Form<T>::ld(src + ((unsigned)a * S + (unsigned)g), a);
+        fs[a] = Form<T>::ld(pdf_at(src, S, a, (unsigned)g), a);
         const unsigned y = at(-cx(a), -cy(a), -cz(a));
         fy[a] = (C)0;
         phy[a] = (C)0;
-        if (ty(a) <= IFC) fy[a] = Form<T>::ld(src + ((unsigned)a * S + y), a);
+        if (ty(a) <= IFC) fy[a] = Form<T>::ld(pdf_at(src, S, a, y), a);
         if (ty(a) == IFC) phy[a] = phic[y];
     }
     const C phx = phic[g];
@@ -1915,8 +1938,8 @@ __device__ __forceinline__ IfOut<typename Form<T>::C> iface_one(const StepArgs& 
     // normals by central differences; the normal test bits of the cell
     const C* __restrict__ nr = (const C*)A.nrm;
     const C dX = nr[at(1, 0, 0)] - nr[at(-1, 0, 0)];
-    const C dY = nr[S + at(0, 1, 0)] - nr[S + at(0, -1, 0)];
-    const C dZ = nr[2u * S + at(0, 0, 1)] - nr[2u * S + at(0, 0, -1)];
+    const C dY = nr[(unsigned)S + at(0, 1, 0)] - nr[(unsigned)S + at(0, -1, 0)];
+    const C dZ = nr[2u * (unsigned)S + at(0, 0, 1)] - nr[2u * (unsigned)S + at(0, 0, -1)];
     const C kappa = (C)0.25 * ((dX + dY) + dZ);
     const unsigned nmk = (unsigned)(link & 0x3ffffu) << 1;   // bit a: the normal test of direction a
     // gas velocity: that of the cell's own post-collision PDFs
@@ -1963,7 +1986,7 @@ __device__ __forceinline__ IfOut<typename Form<T>::C> iface_one(const StepArgs& 
         pair(std::integral_constant<int, 9>{}); pair(std::integral_constant<int, 11>{});
         pair(std::integral_constant<int, 13>{}); pair(std::integral_constant<int, 15>{});
         pair(std::integral_constant<int, 17>{});
-        rho = collide64_any(D.has_force, fin, [&](int a, double v) { dst[(unsigned)a * S + (unsigned)g] = v; }, R.omp,
+        rho = collide64_any(D.has_force, fin, [&](int a, double v) { *pdf_at(dst, S, a, (unsigned)g) = (T)v; }, R.omp,
                             R.omm, R.g);
     } else {
         if constexpr (TWO) {
@@ -2028,13 +2051,13 @@ __device__ __forceinline__ IfOut<typename Form<T>::C> iface_one(const StepArgs& 
             rho = P.rho;
 #pragma unroll
             for (int a = 0; a < 19; ++a)
-                Form<T>::st(dst + ((unsigned)a * S + (unsigned)g), a, collide_out<C, true>(a, fin, P, R.omp, R.omm));
+                Form<T>::st(pdf_at(dst, S, a, (unsigned)g), a, collide_out<C, true>(a, fin, P, R.omp, R.omm));
         } else {
             const CollidePrep<C> P = collide_prep<C, false>(fin, (C)0, (C)0, (C)0);
             rho = P.rho;
 #pragma unroll
             for (int a = 0; a < 19; ++a)
-                Form<T>::st(dst + ((unsigned)a * S + (unsigned)g), a, collide_out<C, false>(a, fin, P, R.omp, R.omm));
+                Form<T>::st(pdf_at(dst, S, a, (unsigned)g), a, collide_out<C, false>(a, fin, P, R.omp, R.omm));
         }
     }
     if (!(rho == rho)) set_status(A.status, ST_NAN);
