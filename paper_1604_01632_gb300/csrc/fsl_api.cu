@@ -209,33 +209,38 @@ cudaError_t staging(fsl_domain* h, const size_t* bytes, int n, void** parts) {
     return cudaSuccess;
 }
 
+bool f64_form(const fsl_domain* h) { return h->precision == FSL_P_FP64; }
+
+// The two-kernel form of the FP32-collide storage forms runs as one tile-fused
+// kernel on lattices of a million cells and more (with its own rounding of the
+// rebuilt PDFs): there the interface cells read what the block has just streamed
+// (256^3 FP32: 1.11 against 1.21 ms of stream-collide work; 64 domains, 15.8 M
+// cells, FP16-s: 0.86 against 0.97 ms).  Below, two kernels are faster.
+bool two_as_tiles(const fsl_domain* h, int f) { return f == SC_TWO && !f64_form(h) && h->stride >= (1LL << 20); }
+bool tile_form(const fsl_domain* h, int f) { return f == SC_TILE2 || f == SC_TILE4 || two_as_tiles(h, f); }
+
+// Kernels one step launches with stream-collide form f: the conversion kernel,
+// plus the normals pass in the forms that take interface cells one per thread,
+// plus one or two stream-collide kernels.
+int kernels_per_step(const fsl_domain* h, int f) {
+    if (tile_form(h, f)) return 3;
+    if (f == SC_TWO || f == SC_TWOC) return 4;
+    return 2;
+}
+
 // Whether the conversion kernel rebuilds the interface list in cell order: by
 // default where the two PDF arrays of a step exceed twice the L2 cache (there
 // an interface cell's neighbour data would otherwise come from DRAM again for
 // every cell that reads it; the rebuild reads the cell types twice).
-// Kernels one step launches with stream-collide form f: the conversion kernel,
-// plus the normals pass in the forms that take interface cells one per thread,
-// plus one or two stream-collide kernels.
-int kernels_per_step(int f) {
-    if (f == SC_TWO || f == SC_TWOC) return 4;
-    if (f == SC_TILE2 || f == SC_TILE4) return 3;
-    return 2;
-}
-
 int order_effective(const fsl_domain* h) {
     if (h->order_mode >= 0) return h->order_mode;
     const double pdf_bytes = 2.0 * 19.0 * (double)h->stride * (double)h->fbytes;
     return h->l2bytes > 0 && pdf_bytes > 2.0 * (double)h->l2bytes ? 1 : 0;
 }
 
-bool f64_form(const fsl_domain* h) { return h->precision == FSL_P_FP64; }
-
-bool tile_form(int f) { return f == SC_TILE2 || f == SC_TILE4; }
-
-// Whether steps of form f leave an interface list behind: the tile-fused forms
-// find their cells themselves, so only the tuning (which runs other forms next)
-// needs one after them.
-bool keeps_list(const fsl_domain* h, int f) { return !tile_form(f) || h->tuning; }
+// Whether steps of form f read an interface list and leave the next one behind:
+// the tile-fused kernels find their cells themselves.
+bool keeps_list(const fsl_domain* h, int f) { return !tile_form(h, f) || h->tuning; }
 
 // form: the stream-collide form of the step (-1: the handle's)
 StepArgs step_args(fsl_domain* h, int src, int form = -1) {
@@ -275,8 +280,9 @@ StepArgs step_args(fsl_domain* h, int src, int form = -1) {
     // cells one per thread, unless phase D has to walk the list anyway to append
     // the next one (two-kernel forms with the list in appended order).
     const int ord = order_effective(h);
-    A.fused = tile_form(form) || ((form == SC_TWO || form == SC_TWOC) && ord) ? 1 : 0;
-    A.order = tile_form(form) ? (keeps_list(h, form) ? 1 : 0) : ord;
+    A.tiled = two_as_tiles(h, form) ? 1 : 0;
+    A.fused = tile_form(h, form) || ((form == SC_TWO || form == SC_TWOC) && ord) ? 1 : 0;
+    A.order = tile_form(h, form) ? (keeps_list(h, form) ? 1 : 0) : ord;
     A.ocnt = h->ocnt;
     A.spins = h->spins;
     A.bar_extra = h->bar_extra;
@@ -427,7 +433,7 @@ int enqueue_main(fsl_domain* h, const StepArgs& A, cudaEvent_t e0, cudaEvent_t e
     if (e1) { record(e1); last_node(1); }
     launch_conv(h, A, h->ls);
     if (phases) cudaEventRecord(next_phase_event(h), h->ls);
-    return kernels_per_step(h->form);
+    return kernels_per_step(h, h->form);
 }
 
 std::pair<cudaEvent_t, cudaEvent_t> next_events(fsl_domain* h) {
@@ -925,6 +931,22 @@ bool form_usable(const fsl_domain* h, int f) {
     return f >= 0 && f < SC_FORMS;
 }
 
+// Forms the tuner may choose.  Where the two-kernel form runs as a tile-fused
+// kernel it is as fast as forms 6 and 7 and differs from them in the last bits of
+// the FP32-collide storage forms, so timing noise would choose between two
+// trajectories.  One of the two families is eligible there: the two-kernel form
+// where its separate kernels were the faster ones (FP32 on single lattices above
+// 6 M cells: 548 against 557 us at 8 M; 16-bit batches above 12 M cells: 954
+// against 959 us at 15.8 M), forms 6 and 7 elsewhere (16-bit single lattices: 782
+// against 819 us at 16.8 M; batches of 2 M cells: 164 against 216 us).
+bool form_eligible(const fsl_domain* h, int f) {
+    const bool two = f == SC_TWO || f == SC_TWOC, tile = f == SC_TILE2 || f == SC_TILE4;
+    if ((!two && !tile) || !two_as_tiles(h, SC_TWO)) return true;
+    const bool wide = h->precision == FSL_P_FP32;
+    const bool prefer_two = h->ndom == 1 ? wide && h->stride >= 6000000 : !wide && h->stride >= 12000000;
+    return prefer_two ? two : tile;
+}
+
 TuneKey tune_key(fsl_domain* h, int icount) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
@@ -963,7 +985,7 @@ fsl_status tune_step(fsl_domain* h) {
     launch_k1(h, A, h->ls, nullptr, nullptr, f);
     CK(h, cudaEventRecord(h->tev[1], h->ls));
     CK(h, launch_conv(h, A, h->ls, f));
-    h->launches += kernels_per_step(f);
+    h->launches += kernels_per_step(h, f);
     h->cur = 1 - h->cur;
     CK(h, cudaEventSynchronize(h->tev[1]));
     float ms = 0.f;
@@ -974,7 +996,7 @@ fsl_status tune_step(fsl_domain* h) {
     if (h->tune_next == kTuneSteps) {
         int best = SC_SPLIT;
         for (int g = 0; g < SC_FORMS; ++g)
-            if (h->tune_ms[g] > 0.0 && h->tune_ms[g] < h->tune_ms[best]) best = g;
+            if (h->tune_ms[g] > 0.0 && h->tune_ms[g] < h->tune_ms[best] && form_eligible(h, g)) best = g;
         h->form = best;
         h->tuning = false;
         h->tune_source = 1;

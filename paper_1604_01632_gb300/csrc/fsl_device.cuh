@@ -124,6 +124,7 @@ struct StepArgs {
     void* phit;                 // fill level as the normal stencil reads it: walls and
                                 // liquid 1, gas 0, interface clamp(phi, 0, 1)
     void* rhoi;                 // density of interface cells at their last collision
+    int tiled;                  // the two-kernel form of this step runs as one tile-fused kernel
     int fused;                  // 1: the interface kernel of this step also forms the fill levels
                                 // and volume terms, and the conversion's phase D takes only the
                                 // cells that a conversion touched
@@ -959,11 +960,7 @@ __device__ __forceinline__ void liquid_single(const StepArgs& A, long long bid) 
 // is dropped).  Both liquid: one 32-bit store per direction.  (Cells 2t and
 // 2t+1 always lie in the same domain: domains start on multiples of 256.)
 template <typename T, bool ONE>
-__device__ __forceinline__ void liquid_pairs(const StepArgs& A, long long bid) {
-    const long long g0 = 2 * (bid * FSL_BLOCK + threadIdx.x);
-    if (g0 >= A.stride) return;
-    const unsigned short ff = *(const unsigned short*)(A.flag + g0);
-    const uint8_t f0 = (uint8_t)(ff & 0xff), f1 = (uint8_t)(ff >> 8);
+__device__ __forceinline__ void liquid_pair(const StepArgs& A, long long g0, uint8_t f0, uint8_t f1) {
     const bool v0 = ctype(f0) == LIQ, v1 = ctype(f1) == LIQ;
     if (!v0 && !v1) return;
     const Dom& D = dom_at<ONE>(A, g0);
@@ -1038,6 +1035,15 @@ __device__ __forceinline__ void liquid_pairs(const StepArgs& A, long long bid) {
         collide_dev2<true>(d, out, R.omp, R.omm, R.g[0], R.g[1], R.g[2]);
     else
         collide_dev2<false>(d, out, R.omp, R.omm, 0.f, 0.f, 0.f);
+}
+
+// The pairs of tile `bid` (512 cells), one per thread of a 256-thread block.
+template <typename T, bool ONE>
+__device__ __forceinline__ void liquid_pairs(const StepArgs& A, long long bid) {
+    const long long g0 = 2 * (bid * FSL_BLOCK + threadIdx.x);
+    if (g0 >= A.stride) return;
+    const unsigned short ff = *(const unsigned short*)(A.flag + g0);
+    liquid_pair<T, ONE>(A, g0, (uint8_t)(ff & 0xff), (uint8_t)(ff >> 8));
 }
 
 // Coordinates of one interface cell, for the 5x5x5 fill-level stencil of the
@@ -1820,15 +1826,19 @@ __device__ inline void warp_add(long long* base, int key, long long v) {
 }
 
 // Rounding of f_eq,a + f_eq,abar = (fp + fm) + (fp - fm) in the FP32-collide
-// two-kernel forms.  fp = wr inn and fm = wr c3 are products, and which of them
-// is fused into its addition decides the last bit of a rebuilt PDF.  These forms
-// have one fixed choice per direction (and storage width, single domain or
-// batch, gas source or normal test), written out here so that a state does not
-// depend on how a compiler arranges the kernel around it:
+// forms that take interface cells one per thread.  fp = wr inn and fm = wr c3 are
+// products, and which of them is fused into its addition decides the last bit of
+// a rebuilt PDF.  Each family of forms has one fixed choice per direction, written
+// out here so that a state does not depend on how a compiler arranges the kernel
+// around it:
 //   u  both products rounded first        p  fp fused in both sums
 //   m  fm fused in both sums              x  fm fused in the first, fp in the second
-// (The tile-fused forms take u for odd and p for even directions, FP64 u.)
-__host__ __device__ constexpr char two_kernel_rounding(int a, bool wide, bool one, bool gas) {
+// The tile-fused forms take u for odd and p for even directions; the two-kernel
+// forms a choice per direction, storage width, single domain or batch, and gas
+// source or normal test.
+enum { IF_TILE = 0, IF_TWO = 1 };
+__host__ __device__ constexpr char rebuild_rounding(int a, int mode, bool wide, bool one, bool gas) {
+    if (mode == IF_TILE) return (a & 1) ? 'u' : 'p';
     const char* t = wide ? (one ? (gas ? "uupupupuxpupupupup" : "uupupupuupupupupup")
                                 : (gas ? "pupuppmpppxpmmmpmp" : "pupuppupppupuuupmp"))
                          : (one ? (gas ? "pupuuupuxpupupupup" : "pupuuupuupupupupup")
@@ -1882,8 +1892,8 @@ template <typename C> struct IfOut {
     int key;          // fused step: bubble of the cell and change of its volume term
     long long dv;
 };
-// TWO: the two-kernel forms (their rounding of the rebuilt PDFs, above).
-template <typename T, bool ONE, bool TWO>
+// MODE: the forms whose rounding of the rebuilt PDFs it takes.
+template <typename T, bool ONE, int MODE>
 __device__ __forceinline__ IfOut<typename Form<T>::C> iface_one(const StepArgs& A, long long g) {
     using C = typename Form<T>::C;
     const Dom& D = dom_at<ONE>(A, g);
@@ -1952,12 +1962,12 @@ __device__ __forceinline__ IfOut<typename Form<T>::C> iface_one(const StepArgs& 
     } else {
         ugx = jsx / rs; ugy = jsy / rs; ugz = jsz / rs;
     }
-    const C usg = ugx * ugx + ugy * ugy + ugz * ugz;
-    const C rg = (C)3 * (pv + R.sigma2 * kappa);
     // stream with bounce-back and reconstruction, then the collision (Eq. 6)
     C fin[19], rho;
     fin[0] = fs[0];
     if constexpr (sizeof(C) == 8) {
+        const C usg = ugx * ugx + ugy * ugy + ugz * ugz;
+        const C rg = (C)3 * (pv + R.sigma2 * kappa);
         // both directions of a pair rebuild from the same sum of equilibria,
         // formed once and only where one of them does
         const double wr1 = weightc<C>(1) * rg, wr2 = weightc<C>(7) * rg, usg15 = 1.5 * usg;
@@ -1989,63 +1999,37 @@ __device__ __forceinline__ IfOut<typename Form<T>::C> iface_one(const StepArgs& 
         rho = collide64_any(D.has_force, fin, [&](int a, double v) { *pdf_at(dst, S, a, (unsigned)g) = (T)v; }, R.omp,
                             R.omm, R.g);
     } else {
-        if constexpr (TWO) {
-            const float us = __fmaf_rn(ugz, ugz, __fmaf_rn(ugx, ugx, __fmul_rn(ugy, ugy)));
-            const float rg2 = __fmul_rn(3.f, __fmaf_rn(R.sigma2, kappa, pv));
-            const float wr1 = __fmul_rn(weightc<float>(1), rg2), wr2 = __fmul_rn(weightc<float>(7), rg2);
-            auto pair = [&](auto ac) {
-                constexpr int a = decltype(ac)::value;
-                const float cu = cdot32<a>(ugx, ugy, ugz), wr = a <= 6 ? wr1 : wr2;
-                const float inn = __fmaf_rn(-1.5f, us, __fmaf_rn(4.5f, __fmul_rn(cu, cu), 1.f)), c3 = __fmul_rn(3.f, cu);
-                auto one = [&](auto kc) {
-                    constexpr int k = decltype(kc)::value;
-                    constexpr char rg_ = two_kernel_rounding(k, sizeof(T) == 4, ONE, true);
-                    constexpr char rn_ = two_kernel_rounding(k, sizeof(T) == 4, ONE, false);
-                    const float own = fs[opp(k)];
-                    const uint8_t t = ty(k);
-                    const float gas = __fsub_rn(feq_both32<rg_>(wr, inn, c3), own);
-                    const float nrm = rg_ == rn_ ? gas : __fsub_rn(feq_both32<rn_>(wr, inn, c3), own);
-                    float v = t == GAS ? gas : fy[k];
-                    if (t < GAS && D.normal_rule && ((nmk >> k) & 1u)) v = nrm;
-                    if (t == OBS) {
-                        v = own;
-                        if (is_lid(k)) v = own + (6.f * weightc<float>(k)) * cdot<float>(k, R.lid[0], R.lid[1], R.lid[2]);
-                    }
-                    fin[k] = v;
-                };
-                one(std::integral_constant<int, a>{});
-                one(std::integral_constant<int, a + 1>{});
-            };
-            pair(std::integral_constant<int, 1>{}); pair(std::integral_constant<int, 3>{});
-            pair(std::integral_constant<int, 5>{}); pair(std::integral_constant<int, 7>{});
-            pair(std::integral_constant<int, 9>{}); pair(std::integral_constant<int, 11>{});
-            pair(std::integral_constant<int, 13>{}); pair(std::integral_constant<int, 15>{});
-            pair(std::integral_constant<int, 17>{});
-        } else {
-#pragma unroll
-            for (int a = 1; a < 19; ++a) {
-                const C fsb = fs[opp(a)];
-                const uint8_t tya = ty(a);
-                if (tya == OBS) {
-                    fin[a] = fsb;
-                    if (is_lid(a)) {
-                        const C cuw = ((C)cx(a) * R.lid[0] + (C)cy(a) * R.lid[1]) + (C)cz(a) * R.lid[2];
-                        fin[a] = fsb + ((C)6 * weightc<C>(a)) * cuw;
-                    }
-                } else {
-                    C fp, fm;
-                    feq_pair<C>(a, rg, ugx, ugy, ugz, usg, fp, fm);
-                    const C fga = (a & 1) ? fp + fm : fp - fm;
-                    const C fgb = (a & 1) ? fp - fm : fp + fm;
-                    if (tya == GAS) {
-                        fin[a] = (fga + fgb) - fsb;
-                    } else {
-                        fin[a] = fy[a];
-                        if (D.normal_rule && ((nmk >> a) & 1u)) fin[a] = (fga + fgb) - fsb;
-                    }
+        const float us = __fmaf_rn(ugz, ugz, __fmaf_rn(ugx, ugx, __fmul_rn(ugy, ugy)));
+        const float rg2 = __fmul_rn(3.f, __fmaf_rn(R.sigma2, kappa, pv));
+        const float wr1 = __fmul_rn(weightc<float>(1), rg2), wr2 = __fmul_rn(weightc<float>(7), rg2);
+        auto pair = [&](auto ac) {
+            constexpr int a = decltype(ac)::value;
+            const float cu = cdot32<a>(ugx, ugy, ugz), wr = a <= 6 ? wr1 : wr2;
+            const float inn = __fmaf_rn(-1.5f, us, __fmaf_rn(4.5f, __fmul_rn(cu, cu), 1.f)), c3 = __fmul_rn(3.f, cu);
+            auto one = [&](auto kc) {
+                constexpr int k = decltype(kc)::value;
+                constexpr char rg_ = rebuild_rounding(k, MODE, sizeof(T) == 4, ONE, true);
+                constexpr char rn_ = rebuild_rounding(k, MODE, sizeof(T) == 4, ONE, false);
+                const float own = fs[opp(k)];
+                const uint8_t t = ty(k);
+                const float gas = __fsub_rn(feq_both32<rg_>(wr, inn, c3), own);
+                const float nrm = rg_ == rn_ ? gas : __fsub_rn(feq_both32<rn_>(wr, inn, c3), own);
+                float v = t == GAS ? gas : fy[k];
+                if (t < GAS && D.normal_rule && ((nmk >> k) & 1u)) v = nrm;
+                if (t == OBS) {
+                    v = own;
+                    if (is_lid(k)) v = own + (6.f * weightc<float>(k)) * cdot<float>(k, R.lid[0], R.lid[1], R.lid[2]);
                 }
-            }
-        }
+                fin[k] = v;
+            };
+            one(std::integral_constant<int, a>{});
+            one(std::integral_constant<int, a + 1>{});
+        };
+        pair(std::integral_constant<int, 1>{}); pair(std::integral_constant<int, 3>{});
+        pair(std::integral_constant<int, 5>{}); pair(std::integral_constant<int, 7>{});
+        pair(std::integral_constant<int, 9>{}); pair(std::integral_constant<int, 11>{});
+        pair(std::integral_constant<int, 13>{}); pair(std::integral_constant<int, 15>{});
+        pair(std::integral_constant<int, 17>{});
         if (D.has_force) {
             const CollidePrep<C> P = collide_prep<C, true>(fin, R.g[0], R.g[1], R.g[2]);
             rho = P.rho;
@@ -2110,7 +2094,7 @@ __global__ void __launch_bounds__(IfThreads<T>::n, sizeof(T) == 8 ? 4 : 5) k_ifa
         long long g = 0;
         if (i < cnt) {
             g = A.ilist[i];
-            o = iface_one<T, ONE, true>(A, g);
+            o = iface_one<T, ONE, IF_TWO>(A, g);
         }
         list_append(A.mlist, A.mcount, o.marked, (int)g);
         if (A.fused) warp_add(A.vfx, o.dv != 0 ? o.key : -1, o.dv);
@@ -2124,10 +2108,17 @@ __device__ inline unsigned ifc_mask16(const uint8_t* flag, long long j);
 // memory (ballot compaction), then processes those one per thread.  The
 // interface cells' neighbour data is what the block has just read, and both
 // kinds of stores to a 32-byte sector meet in L2 before it is written back.
-template <typename T, bool ONE, int TPB>
-__global__ void __launch_bounds__(FSL_BLOCK, 2) k_stream_tile(StepArgs A) {
-    constexpr long long TILE = Form<T>::shifted ? 2 * FSL_BLOCK : FSL_BLOCK;
-    constexpr int SUPER = (int)(TPB * TILE);
+// Threads of a block and blocks per SM: the 16-bit forms' paired collision wants
+// 128 registers (two blocks of 256; 160 x 4 at 96 registers: 6.36 against 6.05 ms
+// on the 512^3 foam), one FP32 cell per thread gets by with 96 and gains from 20
+// warps instead of 16 (256^3 foam: 1.00 against 1.12 ms).
+template <typename T> struct TileBlock {
+    static constexpr int threads = sizeof(T) == 2 ? 256 : 160, blocks = sizeof(T) == 2 ? 2 : 4;
+};
+template <typename T, bool ONE, int TPB, int MODE = IF_TILE>
+__global__ void __launch_bounds__(TileBlock<T>::threads, TileBlock<T>::blocks) k_stream_tile(StepArgs A) {
+    constexpr int NT = TileBlock<T>::threads;
+    constexpr int SUPER = TPB * NT * (Form<T>::shifted ? 2 : 1);
     __shared__ int il[SUPER];
     __shared__ int nil;
     pdl_trigger();   // the conversion kernel may be placed as blocks finish
@@ -2137,15 +2128,25 @@ __global__ void __launch_bounds__(FSL_BLOCK, 2) k_stream_tile(StepArgs A) {
     const long long c0 = (long long)blockIdx.x * SUPER;
 #pragma unroll 1
     for (int k = 0; k < TPB; ++k) {
-        const long long tile = (long long)blockIdx.x * TPB + k;
-        if (tile * TILE >= A.stride) break;
-        if constexpr (Form<T>::shifted) liquid_pairs<T, ONE>(A, tile);
-        else liquid_single<T, ONE>(A, tile);
+        if constexpr (Form<T>::shifted) {
+            const long long g0 = c0 + 2 * (k * NT + (int)threadIdx.x);
+            if (g0 < A.stride) {
+                const unsigned short ff = *(const unsigned short*)(A.flag + g0);
+                liquid_pair<T, ONE>(A, g0, (uint8_t)(ff & 0xff), (uint8_t)(ff >> 8));
+            }
+        } else {
+            const long long g = c0 + k * NT + (int)threadIdx.x;
+            if (g < A.stride) {
+                const uint8_t f = A.flag[g];
+                if (ctype(f) == LIQ) liquid_one<T, ONE>(A, g, f);
+            }
+        }
     }
     // the super-tile's interface cells (a 16-byte load of types per thread)
     const unsigned lane = threadIdx.x & 31u;
-    for (long long j = c0 / 16 + threadIdx.x; j < (c0 + SUPER) / 16; j += FSL_BLOCK) {
-        const unsigned m = j * 16 < A.stride ? ifc_mask16(A.flag, j) : 0u;
+    for (int w0 = 0; w0 < SUPER / 16; w0 += NT) {
+        const long long j = c0 / 16 + w0 + threadIdx.x;
+        const unsigned m = w0 + (int)threadIdx.x < SUPER / 16 && j * 16 < A.stride ? ifc_mask16(A.flag, j) : 0u;
         const int n = __popc(m);
         int incl = n;
 #pragma unroll
@@ -2161,13 +2162,13 @@ __global__ void __launch_bounds__(FSL_BLOCK, 2) k_stream_tile(StepArgs A) {
     }
     __syncthreads();
     const int ni = nil;
-    for (int i0 = 0; i0 < ni; i0 += FSL_BLOCK) {
+    for (int i0 = 0; i0 < ni; i0 += NT) {
         const int i = i0 + threadIdx.x;
         IfOut<typename Form<T>::C> o{false, -1, 0};
         long long g = 0;
         if (i < ni) {
             g = il[i];
-            o = iface_one<T, ONE, false>(A, g);
+            o = iface_one<T, ONE, MODE>(A, g);
         }
         list_append(A.mlist, A.mcount, o.marked, (int)g);
         if (A.fused) warp_add(A.vfx, o.dv != 0 ? o.key : -1, o.dv);
@@ -3678,6 +3679,24 @@ inline void launch_normals(const StepArgs& A, long long nb, cudaStream_t s) {
     }
 }
 
+// The tile-fused kernel of a form (FP64 has none).
+template <typename T>
+inline void launch_tiles(const StepArgs& A, int form, unsigned grid, cudaStream_t s) {
+    if constexpr (sizeof(T) <= 4) {
+        const bool one = A.ndom == 1;
+        if (form == SC_TILE2) {
+            if (one) k_stream_tile<T, true, 2><<<grid, TileBlock<T>::threads, 0, s>>>(A);
+            else k_stream_tile<T, false, 2><<<grid, TileBlock<T>::threads, 0, s>>>(A);
+        } else if (form == SC_TILE4) {
+            if (one) k_stream_tile<T, true, 4><<<grid, TileBlock<T>::threads, 0, s>>>(A);
+            else k_stream_tile<T, false, 4><<<grid, TileBlock<T>::threads, 0, s>>>(A);
+        } else {
+            if (one) k_stream_tile<T, true, 4, IF_TWO><<<grid, TileBlock<T>::threads, 0, s>>>(A);
+            else k_stream_tile<T, false, 4, IF_TWO><<<grid, TileBlock<T>::threads, 0, s>>>(A);
+        }
+    }
+}
+
 // Launch helpers instantiated once per storage form.
 template <typename T> void launch_stream(const StepArgs& A, long long nblocks, int ifblocks, int form, int pgrid,
                                          cudaStream_t s, cudaEvent_t el, cudaEvent_t ei, cudaStream_t s2,
@@ -3709,19 +3728,12 @@ template <typename T> void launch_mass_partials(const void* f, const uint8_t* fl
                 k_stream<T, true><<<(unsigned)(nif + nliq), FSL_BLOCK, 0, s>>>(A, nif);                      \
             else                                                                                             \
                 k_stream<T, false><<<(unsigned)(nif + nliq), FSL_BLOCK, 0, s>>>(A, nif);                     \
-        } else if (form == SC_TILE2 || form == SC_TILE4) {                                                  \
-            const long long tile = Form<T>::shifted ? 2LL * FSL_BLOCK : (long long)FSL_BLOCK;                \
+        } else if (form == SC_TILE2 || form == SC_TILE4 || (form == SC_TWO && A.tiled)) {                                                  \
             const int tpb = form == SC_TILE2 ? 2 : 4;                                                       \
-            const unsigned nsup = (unsigned)((A.stride + tpb * tile - 1) / (tpb * tile));                    \
-            if (A.ndom == 1) {                                                                               \
-                launch_normals<T>(A, nb, s);                                                                 \
-                if (tpb == 2) k_stream_tile<T, true, 2><<<nsup, FSL_BLOCK, 0, s>>>(A);                       \
-                else k_stream_tile<T, true, 4><<<nsup, FSL_BLOCK, 0, s>>>(A);                                \
-            } else {                                                                                         \
-                launch_normals<T>(A, nb, s);                                                                 \
-                if (tpb == 2) k_stream_tile<T, false, 2><<<nsup, FSL_BLOCK, 0, s>>>(A);                      \
-                else k_stream_tile<T, false, 4><<<nsup, FSL_BLOCK, 0, s>>>(A);                               \
-            }                                                                                                \
+            const long long super = (long long)tpb * TileBlock<T>::threads * (Form<T>::shifted ? 2 : 1);                   \
+            const unsigned nsup = (unsigned)((A.stride + super - 1) / super);                                \
+            launch_normals<T>(A, nb, s);                                                                     \
+            launch_tiles<T>(A, form, nsup, s);                                                               \
         } else if (form == SC_TWOC) {                                                                        \
             /* the interface kernel on a second stream, beside the liquid kernel */                          \
             const long long nliq = Form<T>::shifted ? (nb + 1) / 2 : nb;                                     \
@@ -3763,10 +3775,7 @@ template <typename T> void launch_mass_partials(const void* f, const uint8_t* fl
     template <> int stream_blocks_per_sm<T>(int form, bool one) {                                            \
         int nb = 0;                                                                                          \
         if (form == SC_SPLIT) nb = 1;                                                                        \
-        else if (form == SC_TILE2 || form == SC_TILE4) {                                                     \
-            if (one) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_stream_tile<T, true, 2>, FSL_BLOCK, 0); \
-            else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_stream_tile<T, false, 2>, FSL_BLOCK, 0); \
-        }                                                                                                    \
+        else if (form == SC_TILE2 || form == SC_TILE4) nb = 1;                                               \
         else if (form == SC_TWOC && one)                                                                     \
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_iface<T, true>, IfThreads<T>::n, 0);        \
         else if (form == SC_TWOC)                                                                            \
