@@ -1835,26 +1835,25 @@ __device__ inline void warp_add(long long* base, int key, long long v) {
 // a rebuilt PDF.  Each family of forms has one fixed choice per direction, written
 // out here so that a state does not depend on how a compiler arranges the kernel
 // around it:
-//   u  both products rounded first        p  fp fused in both sums
-//   m  fm fused in both sums              x  fm fused in the first, fp in the second
-// The tile-fused forms take u for odd and p for even directions; the two-kernel
+//   p  fp fused in both sums        m  fm fused in both sums
+//   x  fm fused in the first, fp in the second
+// The tile-fused forms take m for odd and p for even directions; the two-kernel
 // forms a choice per direction, storage width, single domain or batch, and gas
 // source or normal test.
 enum { IF_TILE = 0, IF_TWO = 1 };
 __host__ __device__ constexpr char rebuild_rounding(int a, int mode, bool wide, bool one, bool gas) {
-    if (mode == IF_TILE) return (a & 1) ? 'u' : 'p';
-    const char* t = wide ? (one ? (gas ? "uupupupuxpupupupup" : "uupupupuupupupupup")
-                                : (gas ? "pupuppmpppxpmmmpmp" : "pupuppupppupuuupmp"))
-                         : (one ? (gas ? "pupuuupuxpupupupup" : "pupuuupuupupupupup")
-                                : (gas ? "uuupuupppmxpupmpup" : "uuupuupppmupupupup"));
+    if (mode == IF_TILE) return (a & 1) ? 'm' : 'p';
+    const char* t = wide ? (one ? (gas ? "mmpmpmpmxpmpmpmpmp" : "mmpmpmpmmpmpmpmpmp")
+                                : (gas ? "pmpmppmpppxpmmmpmp" : "pmpmppmpppmpmmmpmp"))
+                         : (one ? (gas ? "pmpmmmpmxpmpmpmpmp" : "pmpmmmpmmpmpmpmpmp")
+                                : (gas ? "mmmpmmpppmxpmpmpmp" : "mmmpmmpppmmpmpmpmp"));
     return t[a - 1];
 }
 template <char R>
 __device__ __forceinline__ float feq_both32(float wr, float inn, float c3) {
     const float fp = __fmul_rn(wr, inn), fm = __fmul_rn(wr, c3);
     float plus, minus;
-    if constexpr (R == 'u') { plus = __fadd_rn(fp, fm); minus = __fsub_rn(fp, fm); }
-    else if constexpr (R == 'p') { plus = __fmaf_rn(wr, inn, fm); minus = __fmaf_rn(wr, inn, -fm); }
+    if constexpr (R == 'p') { plus = __fmaf_rn(wr, inn, fm); minus = __fmaf_rn(wr, inn, -fm); }
     else if constexpr (R == 'm') { plus = __fmaf_rn(wr, c3, fp); minus = __fmaf_rn(-wr, c3, fp); }
     else { plus = __fmaf_rn(wr, c3, fp); minus = __fmaf_rn(wr, inn, -fm); }
     return __fadd_rn(plus, minus);
