@@ -218,10 +218,16 @@ fsl_status fsl_set_limits(fsl_domain* h, int64_t ccl_max_iter, int64_t barrier_p
  * the first fsl_step calls of a handle run real steps that each time one
  * candidate form (every usable form twice: the slab form only with the
  * interface list in cell order, the tile-fused forms not in FP64; direct
- * launches, the call waits for each), then keep the fastest and record it in a process-wide cache keyed by
- * precision, one or many domains, SM count, lattice size (log2 of the padded
+ * launches, the call waits for each), then keep the fastest eligible one and
+ * record it in a process-wide cache keyed by precision, one or many domains, SM count, lattice size (log2 of the padded
  * cells) and interface share (1/64 steps); a later handle of the same key
- * takes the cached form without tuning.  Forms:
+ * takes the cached form without tuning.  In FP32 and 16-bit storage the
+ * two-kernel forms 5 and 8 and the tile-fused forms 6 and 7 round the rebuilt
+ * PDFs differently and cost about the same; from 2^20 cells (padded) on only
+ * one of the two pairs is eligible, so that the choice between two
+ * trajectories does not follow timing noise: 5 and 8 in FP32 storage of one
+ * domain of at least 6 million cells and in 16-bit batches of at least 12
+ * million, 6 and 7 otherwise.  Forms:
  *   0  split: blocks [0, 2 x SMs) take the interface list in 32-cell chunks
  *      (16 in FP64), the other blocks one liquid tile each;
  *   1, 2, 3  persistent: a resident grid walks one sequence of work items in
@@ -232,7 +238,9 @@ fsl_status fsl_set_limits(fsl_domain* h, int64_t ccl_max_iter, int64_t barrier_p
  *      interleaved (only with the interface list in cell order, see
  *      fsl_set_interface_order; FSL_ERR_ARG otherwise);
  *   5  two kernels: the liquid cells (a tile per block), then the interface
- *      cells one per thread with every direction unrolled;
+ *      cells one per thread with every direction unrolled.  From 2^20 cells
+ *      on, in FP32 and 16-bit storage, the same cells with the same results
+ *      by one tile-fused kernel (4 tiles per block);
  *   6, 7  tile-fused: each block takes 2 or 4 tiles, streams and collides
  *      their liquid cells, then their interface cells one per thread (FP32
  *      and 16-bit storage only; FSL_ERR_ARG for FP64);
@@ -243,7 +251,10 @@ fsl_status fsl_set_limits(fsl_domain* h, int64_t ccl_max_iter, int64_t barrier_p
  * stores the unit normal of every interface cell and face neighbour of one
  * and each interface cell's reconstruction directions; their interface cells
  * read the curvature's normals from it.  Kernels per step: 4 in forms 5 and
- * 8, 3 in forms 6 and 7, 2 otherwise (the conversion kernel included).
+ * 8, 3 in forms 6 and 7 and in form 5 where it is tile-fused, 2 otherwise (the
+ * conversion kernel included).  The tile-fused kernels find their interface
+ * cells themselves: no interface list is kept while they run, and the first
+ * step of another form rebuilds it.
  * -1 restarts the tuning.  Waits for the handle's stream; the next fsl_step
  * rebuilds its graphs.  FSL_ERR_ARG for another value.  fsl_stream_form
  * returns the form in use (the one tried next while tuning). */
