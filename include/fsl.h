@@ -213,21 +213,20 @@ fsl_status fsl_set_graphs(fsl_domain* h, int32_t on);
  * FSL_ERR_ARG for values out of range. */
 fsl_status fsl_set_limits(fsl_domain* h, int64_t ccl_max_iter, int64_t barrier_polls, int32_t barrier_absent);
 
-/* Form of the stream-collide kernel (the same results in every form; each
- * cell runs the same arithmetic).  By default (form -1) the library tunes it:
- * the first fsl_step calls of a handle run real steps that each time one
- * candidate form (every usable form twice: the slab form only with the
- * interface list in cell order, the tile-fused forms not in FP64; direct
- * launches, the call waits for each), then keep the fastest eligible one and
- * record it in a process-wide cache keyed by precision, one or many domains, SM count, lattice size (log2 of the padded
- * cells) and interface share (1/64 steps); a later handle of the same key
- * takes the cached form without tuning.  In FP32 and 16-bit storage the
- * two-kernel forms 5 and 8 and the tile-fused forms 6 and 7 round the rebuilt
- * PDFs differently and cost about the same; from 2^20 cells (padded) on only
- * one of the two pairs is eligible, so that the choice between two
- * trajectories does not follow timing noise: 5 and 8 in FP32 storage of one
- * domain of at least 6 million cells and in 16-bit batches of at least 12
- * million, 6 and 7 otherwise.  Forms:
+/* Form of the stream-collide kernel.  FP64 storage gives the same state, bit
+ * for bit, in every form.  In FP32 and 16-bit storage the forms fall into three
+ * families, 0-4, 5 and 8, 6 and 7: the same state bit for bit within a family,
+ * another rounding (of the PDFs rebuilt at the interface) in each.  By default
+ * (form -1) the library tunes the form: the first fsl_step calls of a handle
+ * run real steps that each time one candidate form (every usable form twice:
+ * the slab form only with the interface list in cell order, the tile-fused
+ * forms not in FP64; direct launches, the call waits for each), then keep the
+ * fastest and record it in a process-wide cache keyed by precision, one or many
+ * domains, SM count, lattice size (log2 of the padded cells) and interface
+ * share (1/64 steps); a later handle of the same key takes the cached form
+ * without tuning.  In FP32 and 16-bit storage the fastest of one family is
+ * kept, and that family is a function of the key alone (family_of in
+ * csrc/fsl_forms.h), so that no timing decides between two roundings.  Forms:
  *   0  split: blocks [0, 2 x SMs) take the interface list in 32-cell chunks
  *      (16 in FP64), the other blocks one liquid tile each;
  *   1, 2, 3  persistent: a resident grid walks one sequence of work items in

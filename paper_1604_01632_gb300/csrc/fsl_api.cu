@@ -32,19 +32,7 @@ const int kTuneSeq[] = {SC_SPLIT, SC_PERS1, SC_PERS2, SC_PERS4, SC_SLAB, SC_TWO,
                         SC_SPLIT, SC_PERS1, SC_PERS2, SC_PERS4, SC_SLAB, SC_TWO, SC_TILE2, SC_TILE4, SC_TWOC};
 const int kTuneSteps = (int)(sizeof(kTuneSeq) / sizeof(kTuneSeq[0]));
 
-// Process-wide cache of tuning decisions, keyed by the workload's shape:
-// storage precision, one or many domains, SM count, lattice size (log2 of the
-// padded cells) and the interface share (in 1/64 steps) at tuning time.
-struct TuneKey {
-    int prec, multi, sms, lsize, ifrac;
-    bool operator<(const TuneKey& o) const {
-        if (prec != o.prec) return prec < o.prec;
-        if (multi != o.multi) return multi < o.multi;
-        if (sms != o.sms) return sms < o.sms;
-        if (lsize != o.lsize) return lsize < o.lsize;
-        return ifrac < o.ifrac;
-    }
-};
+// Process-wide cache of tuning decisions.
 std::mutex g_tune_mutex;
 std::map<TuneKey, int> g_tune_cache;
 
@@ -931,22 +919,6 @@ bool form_usable(const fsl_domain* h, int f) {
     return f >= 0 && f < SC_FORMS;
 }
 
-// Forms the tuner may choose.  Where the two-kernel form runs as a tile-fused
-// kernel it is as fast as forms 6 and 7 and differs from them in the last bits of
-// the FP32-collide storage forms, so timing noise would choose between two
-// trajectories.  One of the two families is eligible there: the two-kernel form
-// where its separate kernels were the faster ones (FP32 on single lattices above
-// 6 M cells: 548 against 557 us at 8 M; 16-bit batches above 12 M cells: 954
-// against 959 us at 15.8 M), forms 6 and 7 elsewhere (16-bit single lattices: 782
-// against 819 us at 16.8 M; batches of 2 M cells: 164 against 216 us).
-bool form_eligible(const fsl_domain* h, int f) {
-    const bool two = f == SC_TWO || f == SC_TWOC, tile = f == SC_TILE2 || f == SC_TILE4;
-    if ((!two && !tile) || !two_as_tiles(h, SC_TWO)) return true;
-    const bool wide = h->precision == FSL_P_FP32;
-    const bool prefer_two = h->ndom == 1 ? wide && h->stride >= 6000000 : !wide && h->stride >= 12000000;
-    return prefer_two ? two : tile;
-}
-
 TuneKey tune_key(fsl_domain* h, int icount) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
@@ -958,7 +930,8 @@ TuneKey tune_key(fsl_domain* h, int icount) {
 
 // One autotuning step: the next candidate form, its stream-collide kernel
 // bracketed by events and timed (the call waits for it).  After the last
-// candidate the fastest form is kept and recorded in the process cache.
+// candidate the fastest form of the workload's family is kept and recorded in the
+// process cache.
 fsl_status tune_step(fsl_domain* h) {
     if (h->tune_next == 0) {
         int ic = 0;
@@ -994,17 +967,17 @@ fsl_status tune_step(fsl_domain* h) {
     ++h->tune_next;
     while (h->tune_next < kTuneSteps && !form_usable(h, kTuneSeq[h->tune_next])) ++h->tune_next;
     if (h->tune_next == kTuneSteps) {
-        int best = SC_SPLIT;
-        for (int g = 0; g < SC_FORMS; ++g)
-            if (h->tune_ms[g] > 0.0 && h->tune_ms[g] < h->tune_ms[best] && form_eligible(h, g)) best = g;
-        h->form = best;
-        h->tuning = false;
-        h->tune_source = 1;
         int ic = 0;
         CK(h, cudaMemcpyAsync(&ic, h->icount[h->cur], sizeof(int), cudaMemcpyDeviceToHost, h->ls));
         CK(h, cudaStreamSynchronize(h->ls));
+        const TuneKey key = tune_key(h, ic);
+        bool usable[SC_FORMS];
+        for (int g = 0; g < SC_FORMS; ++g) usable[g] = form_usable(h, g);
+        h->form = choose_form(key, h->tune_ms, usable);
+        h->tuning = false;
+        h->tune_source = 1;
         std::lock_guard<std::mutex> lock(g_tune_mutex);
-        g_tune_cache[tune_key(h, ic)] = best;
+        g_tune_cache[key] = h->form;
         drop_graphs(h);
     }
     return FSL_OK;

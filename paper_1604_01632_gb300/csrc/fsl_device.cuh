@@ -22,6 +22,8 @@
 
 #include <type_traits>
 
+#include "fsl_forms.h"
+
 #define FSL_BLOCK 256
 #define FSL_CONV_THREADS 256   // block of the cooperative conversion kernel
 
@@ -2296,15 +2298,6 @@ __global__ void __launch_bounds__(FSL_BLOCK, sizeof(T) == 8 ? 2 : FSL_STREAM_MIN
         }
     }
 }
-
-// Stream-collide kernel forms (the autotuner picks one per workload): the split
-// form (interface blocks first, then one block per liquid tile), the
-// persistent form with 1, 2 or 4 tiles per liquid item, the slab form, the
-// two-kernel form (liquid kernel, then one thread per interface cell), the
-// tile-fused form with 2 or 4 tiles per block, and the two kernels run side by
-// side on two streams.
-enum { SC_SPLIT = 0, SC_PERS1 = 1, SC_PERS2 = 2, SC_PERS4 = 3, SC_SLAB = 4, SC_TWO = 5, SC_TILE2 = 6, SC_TILE4 = 7,
-       SC_TWOC = 8, SC_FORMS = 9 };
 
 // The neighbour scans below load all eighteen neighbours first and then test
 // them (one memory latency, not one per neighbour): bit a of the mask is set
