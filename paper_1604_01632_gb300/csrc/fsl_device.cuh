@@ -2658,7 +2658,10 @@ __device__ inline void mark_affected(const StepArgs& A, const CclArgs& K, int d,
 }
 
 // Unit normal n = -g / |g| of the fill level at cell w (Parker-Youngs gradient
-// g over the 3x3x3 stencil of the stencil fill levels), 0 where g = 0.
+// g over the 3x3x3 stencil of the stencil fill levels), 0 where g = 0.  The levels
+// are those of the start of the step in every stream-collide form: from the types,
+// which phase D changes only later, and the fill levels the step started from (in a
+// fused step the interface kernel has already replaced the stored stencil levels).
 template <typename C>
 __device__ inline void unit_normal_at(const StepArgs& A, const Dom& D, long long w, float& nx, float& ny, float& nz) {
     const Cell c = make_cell(D, w);
@@ -2666,7 +2669,9 @@ __device__ inline void unit_normal_at(const StepArgs& A, const Dom& D, long long
 #pragma unroll
     for (int k = 0; k < 27; ++k) {
         const long long z = c.at(k % 3 - 1, (k / 3) % 3 - 1, k / 9 - 1);
-        v[k] = (float)((const C*)A.phit)[z];
+        const uint8_t t = ctype(A.flag[z]);
+        const float ph = (float)clamp01(((const C*)A.phi)[z]);
+        v[k] = t == IFC ? ph : (t == GAS ? 0.f : 1.f);
     }
     float gx = 0.f, gy = 0.f, gz = 0.f;
 #pragma unroll
