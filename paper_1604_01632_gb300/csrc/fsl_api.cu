@@ -928,11 +928,17 @@ TuneKey tune_key(fsl_domain* h, int icount) {
     return TuneKey{h->precision, h->ndom > 1 ? 1 : 0, sms, lsize, (int)(64LL * icount / std::max(1LL, h->stride))};
 }
 
+void usable_forms(const fsl_domain* h, bool* usable) {
+    for (int f = 0; f < SC_FORMS; ++f) usable[f] = form_usable(h, f);
+}
+
 // One autotuning step: the next candidate form, its stream-collide kernel
 // bracketed by events and timed (the call waits for it).  After the last
 // candidate the fastest form of the workload's family is kept and recorded in the
 // process cache.
 fsl_status tune_step(fsl_domain* h) {
+    bool usable[SC_FORMS];
+    usable_forms(h, usable);
     if (h->tune_next == 0) {
         int ic = 0;
         CK(h, cudaMemcpyAsync(&ic, h->icount[h->cur], sizeof(int), cudaMemcpyDeviceToHost, h->ls));
@@ -941,13 +947,13 @@ fsl_status tune_step(fsl_domain* h) {
         std::lock_guard<std::mutex> lock(g_tune_mutex);
         auto it = g_tune_cache.find(key);
         if (it != g_tune_cache.end()) {
-            h->form = it->second;
+            h->form = cached_form(it->second, usable);
             h->tuning = false;
             h->tune_source = 2;
             return FSL_OK;   // no step taken: the caller runs it with the cached form
         }
     }
-    while (h->tune_next < kTuneSteps && !form_usable(h, kTuneSeq[h->tune_next])) ++h->tune_next;
+    while (h->tune_next < kTuneSteps && !usable[kTuneSeq[h->tune_next]]) ++h->tune_next;
     const int f = kTuneSeq[h->tune_next];
     if (!h->tev[0]) {
         CK(h, cudaEventCreate(&h->tev[0]));
@@ -965,14 +971,12 @@ fsl_status tune_step(fsl_domain* h) {
     CK(h, cudaEventElapsedTime(&ms, h->tev[0], h->tev[1]));
     if (h->tune_ms[f] == 0.0 || ms < h->tune_ms[f]) h->tune_ms[f] = ms;
     ++h->tune_next;
-    while (h->tune_next < kTuneSteps && !form_usable(h, kTuneSeq[h->tune_next])) ++h->tune_next;
+    while (h->tune_next < kTuneSteps && !usable[kTuneSeq[h->tune_next]]) ++h->tune_next;
     if (h->tune_next == kTuneSteps) {
         int ic = 0;
         CK(h, cudaMemcpyAsync(&ic, h->icount[h->cur], sizeof(int), cudaMemcpyDeviceToHost, h->ls));
         CK(h, cudaStreamSynchronize(h->ls));
         const TuneKey key = tune_key(h, ic);
-        bool usable[SC_FORMS];
-        for (int g = 0; g < SC_FORMS; ++g) usable[g] = form_usable(h, g);
         h->form = choose_form(key, h->tune_ms, usable);
         h->tuning = false;
         h->tune_source = 1;

@@ -84,4 +84,10 @@ inline int choose_form(const TuneKey& k, const double* ms, const bool* usable) {
     return best >= 0 ? best : first;
 }
 
+// The form a handle takes from the cache.  The key does not hold the order of the
+// interface list, which an option sets per handle and which the slab form needs: a
+// handle with the list in appended order takes the split form, of the same family,
+// in its place.
+inline int cached_form(int form, const bool* usable) { return usable[form] ? form : SC_SPLIT; }
+
 }  // namespace fsl

@@ -19,6 +19,7 @@ extern "C" int family_of_form(int form) { return form_family(form); }
 extern "C" int choose(int prec, int multi, int lsize, int ifrac, const double* ms, const bool* usable) {
     return choose_form(TuneKey{prec, multi, 152, lsize, ifrac}, ms, usable);
 }
+extern "C" int cached(int form, const bool* usable) { return cached_form(form, usable); }
 """
 
 
@@ -63,3 +64,15 @@ def test_the_choice_stays_in_the_family_of_the_key(lib):
     ((FP32, 1, 18, 8), 6), ((FP32, 1, 23, 8), 6)])
 def test_the_families_on_either_side_of_each_line(lib, key, first):
     assert lib.family(*key) == lib.family_of_form(first)
+
+
+def test_a_cached_slab_form_needs_the_ordered_list(lib):
+    """A handle whose interface list is in appended order does not take the slab form
+    that another handle of the same key left in the cache: it searches the list."""
+    for order in (False, True):
+        usable = (ctypes.c_bool * FORMS)(*[True] * FORMS)
+        usable[4] = order
+        for form in range(FORMS):
+            got = lib.cached(form, usable)
+            assert usable[got] and lib.family_of_form(got) == lib.family_of_form(form)
+            assert got == form or (form == 4 and not order)
