@@ -1003,21 +1003,25 @@ __device__ __forceinline__ void liquid_pair(const StepArgs& A, long long g0, uin
         if (!(D.nx & 1)) pull(std::true_type{});
         else pull(std::false_type{});
     } else {
-        const Pull P0 = make_pull(D, g0), P1 = make_pull(D, g0 + 1);
         // walls, or a pair that straddles two rows: every link of each cell on
-        // its own, a wall cell's bounced links chosen without a branch
+        // its own, a wall cell's bounced links chosen without a branch.  (After
+        // the last cell of a domain of odd size the second cell is padding, which
+        // no coordinate describes: a second lane that is not liquid repeats the
+        // first one's loads.)
+        const Pull P0 = make_pull(D, g0), P1 = v1 ? make_pull(D, g0 + 1) : P0;
+        const unsigned g1 = v1 ? gi + 1u : gi;
         const bool k0 = v0 && (f0 & K_WALL), k1 = v1 && (f1 & K_WALL);
-        d[0] = make_float2(Form<T>::ld_dev(pdf_at(src, S, 0, gi)), Form<T>::ld_dev(pdf_at(src, S, 0, gi + 1u)));
+        d[0] = make_float2(Form<T>::ld_dev(pdf_at(src, S, 0, gi)), Form<T>::ld_dev(pdf_at(src, S, 0, g1)));
 #pragma unroll
         for (int a = 1; a < 19; ++a) {
             const unsigned y0 = gi + (unsigned)(P0.ox[1 - cx(a)] + P0.oy[1 - cy(a)] + P0.oz[1 - cz(a)]);
-            const unsigned y1 = gi + 1u + (unsigned)(P1.ox[1 - cx(a)] + P1.oy[1 - cy(a)] + P1.oz[1 - cz(a)]);
+            const unsigned y1 = g1 + (unsigned)(P1.ox[1 - cx(a)] + P1.oy[1 - cy(a)] + P1.oz[1 - cz(a)]);
             const uint8_t t0 = k0 ? ctype(A.flag[y0]) : (uint8_t)LIQ;
             const uint8_t t1 = k1 ? ctype(A.flag[y1]) : (uint8_t)LIQ;
             // bounce-back reads the cell's own opposite PDF (w_a = w_abar)
             const bool b0 = t0 == OBS || t0 == LID, b1 = t1 == OBS || t1 == LID;
             float x0 = Form<T>::ld_dev(b0 ? pdf_at(src, S, opp(a), gi) : pdf_at(src, S, a, y0));
-            float x1 = Form<T>::ld_dev(b1 ? pdf_at(src, S, opp(a), gi + 1u) : pdf_at(src, S, a, y1));
+            float x1 = Form<T>::ld_dev(b1 ? pdf_at(src, S, opp(a), g1) : pdf_at(src, S, a, y1));
             const float lidt = (6.f * weightc<float>(a)) * cdot<float>(a, R.lid[0], R.lid[1], R.lid[2]);
             if (t0 == LID) x0 += lidt;
             if (t1 == LID) x1 += lidt;
