@@ -3546,9 +3546,8 @@ __device__ __forceinline__ double to_double(float x) {
     return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
 }
 
-// Error-free running sum in two FP32 words (Knuth's two-sum): s + e is the
-// exact sum while the errors fit one word, which they do for distributions
-// (terms below 1 in steps of 2^-31 or so; the FP64 sum of them is exact too).
+// Running sum in two FP32 words (Knuth's two-sum): s + e is the exact sum while
+// the errors fit one word.
 struct Sum2 {
     float s, e;
     __device__ __forceinline__ explicit Sum2(float x) : s(x), e(0.f) {}
@@ -3557,24 +3556,43 @@ struct Sum2 {
         e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, v)), __fsub_rn(x, v)));
         s = t;
     }
+    // s: the sum rounded to FP32, e: the rest (after a cancellation s is as small as
+    // the errors collected in e)
+    __device__ __forceinline__ void settle() {
+        const float x = e;
+        e = 0.f;
+        add(x);
+    }
     __device__ __forceinline__ double value() const { return to_double(s) + to_double(e); }
 };
 
 // Density and velocity (Eqs. 4-5) of FP32 distributions as FP64 values.  The
 // plain form (moments and three divisions in FP64, after 19 conversions) costs
-// about 95 operations of the FP64 pipe a cell and is bound by it: 25 ms of the
-// 30 ms read-back of a 512^3 lattice.  Here the sums run in FP32 pairs, and a
+// about 95 operations of the FP64 pipe a cell and is bound by it: nearly all of the
+// 28 ms read-back of a 512^3 lattice.  Here the sums run in FP32 pairs, and a
 // quotient j / r is an FP32 quotient q corrected once in FP64, q + (j - r q) y,
-// with y = 1 / r after one Newton step (46 bits; j - r q is below 2^-22 j, so y
-// adds no error to the rounded result): 12 FP64 operations a cell.  Measured, the
-// whole read-back of types, fill levels, density and velocity: 512^3 FP16-s 30.1 ->
-// 7.1 ms, 256^3 FP32 3.85 -> 0.97 ms.
+// with y = 1 / r after two Newton steps (j - r q is below 2^-22 j, so y adds no
+// error to the rounded result): 14 FP64 operations a cell.  The sums are exact, as
+// those of the plain form are, where the largest and the smallest magnitude among
+// the terms are less than 2^15 apart: the terms are multiples of 2^-39 of the
+// largest, and the nineteen errors add up to less than 2^-16 of it, so e has less
+// than 2^24 steps.  Other cells (a velocity at which one equilibrium is nearly
+// zero) take the plain form.  Measured, the whole read-back of types, fill levels,
+// density and velocity: 512^3 FP16-s 27.8 -> 5.7 ms, 256^3 FP32 3.51 -> 0.76 ms (one
+// Newton step, with which a velocity in some 30,000 misses the rounded quotient by an
+// ulp: 5.2 and 0.69 ms).
 __device__ __forceinline__ void moments_wide(const float* f, double& rho, double& ux, double& uy, double& uz) {
     Sum2 r(f[0]);
+    float lo = fabsf(f[0]), hi = lo;
 #pragma unroll
-    for (int a = 1; a < 19; ++a) r.add(f[a]);
+    for (int a = 1; a < 19; ++a) {
+        r.add(f[a]);
+        lo = fminf(lo, fabsf(f[a]));
+        hi = fmaxf(hi, fabsf(f[a]));
+    }
+    r.settle();
     const float rf = fabsf(r.s);
-    if (rf > 1e-18f && rf < 1e18f) {
+    if (rf >= hi && hi > 1e-18f && rf < 1e18f && lo * 32768.f >= hi) {
         Sum2 jx(f[1]), jy(f[3]), jz(f[5]);
 #pragma unroll
         for (int a = 2; a < 19; ++a) {
@@ -3584,15 +3602,16 @@ __device__ __forceinline__ void moments_wide(const float* f, double& rho, double
         }
         rho = r.value();
         const float y0f = __frcp_rn(r.s);
-        const double y0 = to_double(y0f), y = fma(y0, fma(-rho, y0, 1.0), y0);
-        auto quotient = [&](const Sum2& j) {
+        const double y0 = to_double(y0f), y1 = fma(y0, fma(-rho, y0, 1.0), y0), y = fma(y1, fma(-rho, y1, 1.0), y1);
+        auto quotient = [&](Sum2& j) {
+            j.settle();
             const double q = to_double(__fmul_rn(j.s, y0f));
             return fma(fma(-rho, q, j.value()), y, q);
         };
         ux = quotient(jx); uy = quotient(jy); uz = quotient(jz);
         return;
     }
-    // nothing there (all zero: cells that never held liquid), or out of range
+    // nothing there (all zero: cells that never held liquid), or out of that range
     double fo[19], j[3];
     bool zero = true;
 #pragma unroll
