@@ -34,8 +34,8 @@ namespace fsl {
 enum : uint8_t { LIQ = 0, IFC = 1, GAS = 2, OBS = 3, LID = 4 };
 enum : uint8_t { K_TYPE = 7, K_WALL = 8 };
 __host__ __device__ inline uint8_t ctype(uint8_t f) { return (uint8_t)(f & K_TYPE); }
-// Conversion marks (paper Sec. 2.2, cell conversion).  K1 writes NONE /
-// FILLED / EMPTIED on interface cells; phase A writes NEWG on gas cells and
+// Conversion marks (paper Sec. 2.2, cell conversion), NONE between steps.  The
+// interface kernels write FILLED / EMPTIED on interface cells; phase A writes NEWG on gas cells and
 // clears EMPTIED next to FILLED; phase B writes NEWL / NONE on liquid cells;
 // phase C turns FILLED / EMPTIED into CFILLED / CEMPTIED (same meaning).
 enum : uint8_t { MK_NONE = 0, MK_FILLED = 1, MK_EMPTIED = 2, MK_NEWG = 3, MK_NEWL = 4,
@@ -1633,8 +1633,8 @@ __device__ inline unsigned long long link_kinds(const Pull& P, const uint8_t* fl
 // reconstruction's normal test (Eq. 11) uses the gradient at x itself.  Each
 // normal is computed here once, for every cell that is an interface cell or a
 // face neighbour of one (walls included: the stencil reads walls as full), and
-// stored in nrm; each interface cell also stores its 18 link word in
-// links, and the pressure of its bubble (Eq. 13) in pvc.  The stencil values
+// stored in nrm; each interface cell also stores its link word (the normal test
+// and the kind of its sources) in links, and the pressure of its bubble (Eq. 13) in pvc.  The stencil values
 // are the stored copy phit (walls and liquid 1, gas 0, interface clamp(phi, 0,
 // 1)) and the arithmetic is that of the interface kernels, so their curvature
 // and reconstruction come out as if they had computed the normals themselves.
@@ -1845,7 +1845,10 @@ __device__ inline void warp_add(long long* base, int key, long long v) {
 //   x  fm fused in the first, fp in the second
 // The tile-fused forms take m for odd and p for even directions; the two-kernel
 // forms a choice per direction, storage width, single domain or batch, and gas
-// source or normal test.
+// source or normal test.  No choice is more accurate than another (each rounds one of
+// the two products, then the sum); these are the ones that either family's states have
+// always had, and another would move a chaotic flow to another state.
+// Which family a workload runs is family_of's rule (fsl_forms.h).
 enum { IF_TILE = 0, IF_TWO = 1 };
 __host__ __device__ constexpr char rebuild_rounding(int a, int mode, bool wide, bool one, bool gas) {
     if (mode == IF_TILE) return (a & 1) ? 'm' : 'p';
@@ -1880,12 +1883,12 @@ __device__ __forceinline__ float cdot32(float vx, float vy, float vz) {
     }
 }
 
-// One interface cell g by one thread, every direction unrolled: the same
-// steps and the same arithmetic, operation by operation, as the shared
-// interface pass (stream with bounce-back, Eq. 7; mass exchange over the 18
+// One interface cell g by one thread, every direction unrolled: the steps of the
+// shared interface pass (stream with bounce-back, Eq. 7; mass exchange over the 18
 // links in direction order, Eq. 10; reconstruction from the bubble's gas
 // density 3 (p_V + 2 sigma kappa), Eqs. 8, 11-15; collision, Eq. 6; filled /
-// emptied marks).  The curvature and the normal test come from the normals
+// emptied marks), in FP64 with the same values, in the FP32-collide forms with its
+// own rounding of the rebuilt PDFs.  The curvature and the normal test come from the normals
 // pass (k_normals), run before this kernel in the same step.
 //
 // In a fused step the cell also takes its new fill level phi = m / rho (Eq. 9)
