@@ -222,11 +222,12 @@ fsl_status fsl_set_limits(fsl_domain* h, int64_t ccl_max_iter, int64_t barrier_p
  * the slab form only with the interface list in cell order, the tile-fused
  * forms not in FP64; direct launches, the call waits for each), then keep the
  * fastest and record it in a process-wide cache keyed by precision, one or many
- * domains, SM count, lattice size (log2 of the padded cells) and interface
- * share (1/64 steps); a later handle of the same key takes the cached form
+ * domains, SM count, lattice size (log2 of the padded cells), interface share
+ * (1/64 steps) and family; a later handle of the same key takes the cached form
  * without tuning.  In FP32 and 16-bit storage the fastest of one family is
- * kept, and that family is a function of the key alone (family_of in
- * csrc/fsl_forms.h), so that no timing decides between two roundings.  Forms:
+ * kept, and that family is a function of the precision, one or many domains,
+ * the cells and the interface share (family_of in csrc/fsl_forms.h), so that no
+ * timing decides between two roundings.  Forms:
  *   0  split: blocks [0, 2 x SMs) take the interface list in 32-cell chunks
  *      (16 in FP64), the other blocks one liquid tile each;
  *   1, 2, 3  persistent: a resident grid walks one sequence of work items in

@@ -923,9 +923,7 @@ TuneKey tune_key(fsl_domain* h, int icount) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int lsize = 0;
-    while ((1LL << (lsize + 1)) <= h->stride) ++lsize;
-    return TuneKey{h->precision, h->ndom > 1 ? 1 : 0, sms, lsize, (int)(64LL * icount / std::max(1LL, h->stride))};
+    return TuneKey(h->precision, h->ndom > 1, sms, h->stride, icount);
 }
 
 void usable_forms(const fsl_domain* h, bool* usable) {

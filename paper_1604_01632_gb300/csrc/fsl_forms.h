@@ -15,20 +15,6 @@ namespace fsl {
 enum { SC_SPLIT = 0, SC_PERS1 = 1, SC_PERS2 = 2, SC_PERS4 = 3, SC_SLAB = 4, SC_TWO = 5, SC_TILE2 = 6, SC_TILE4 = 7,
        SC_TWOC = 8, SC_FORMS = 9 };
 
-// A tuning decision holds for one shape of workload: storage precision, one or
-// many domains, SM count, lattice size (floor of log2 of the padded cells) and
-// the interface cells among them (in 1/64).
-struct TuneKey {
-    int prec, multi, sms, lsize, ifrac;
-    bool operator<(const TuneKey& o) const {
-        if (prec != o.prec) return prec < o.prec;
-        if (multi != o.multi) return multi < o.multi;
-        if (sms != o.sms) return sms < o.sms;
-        if (lsize != o.lsize) return lsize < o.lsize;
-        return ifrac < o.ifrac;
-    }
-};
-
 // In FP32 and 16-bit storage the forms fall into three families that round the
 // PDFs rebuilt at the interface differently in the last bit (in FP64 every form
 // gives the same bits).  A chaotic flow makes another state of that bit within
@@ -41,11 +27,11 @@ inline int form_family(int form) {
     return form == SC_TILE2 || form == SC_TILE4 ? FAM_TILE : FAM_SHARED;
 }
 
-// The family the tuner chooses from, a function of the key alone: no timing, and
-// nothing that ran before in the process, enters it.  The lines are where the
+// The family the tuner chooses from: a function of the storage precision, one or many
+// domains, the padded cells and the interface cells among them (in 1/64).  No timing,
+// and nothing that ran before in the process, enters it.  The lines are where the
 // fastest form of one family became that of another when each family still had a
-// kernel of its own, so that a workload stays on the states it has had; they lie on
-// bounds of the key, so that one cached form serves the whole key.
+// kernel of its own, so that a workload stays on the states it has had.
 // Stream-collide work of a step at the lines (us, fastest form of each family,
 // SHARED / TWO / TILE; one domain unless said otherwise):
 //   few interface cells: FP16-s 1.4 M cells, 1.7/64 interface  51 /  63 /  76
@@ -57,27 +43,49 @@ inline int form_family(int form) {
 //                               285 k cells, 8.3/64             36 /  28 /  29
 //   TWO against TILE (equal since both run as the same tile-fused kernel):
 //                        FP32   3.4 M cells, 5.5/64            240 / 207 / 207
-//                               8.4 M cells, 5.7/64            624 / 490 / 490
+//                               3.0 M cells, 7.0/64            254 / 193 / 193
 //                        batch, FP16-s 15.8 M cells, 8.1/64   1830 / 857 / 838
-inline int family_of(const TuneKey& k) {
-    const bool wide = k.prec == FSL_P_FP32;
-    // largest lattice (log2) whose interface work, at that share of the cells, forms
-    // 0-4 still hide behind the liquid tiles of the same launch
-    int shared_up_to = !wide && k.multi ? 16 : 17;
-    if (k.ifrac < 5) shared_up_to = wide ? 22 : 20;
-    if (k.ifrac < 3) shared_up_to = wide ? 63 : 23;
-    if (k.ifrac < 2) shared_up_to = 63;
-    if (k.lsize <= shared_up_to) return FAM_SHARED;
-    if (wide) return !k.multi && k.lsize >= 22 ? FAM_TWO : FAM_TILE;
-    return k.multi && k.lsize >= 23 ? FAM_TWO : FAM_TILE;
+inline int family_of(int prec, bool multi, long long cells, int ifrac) {
+    const bool wide = prec == FSL_P_FP32;
+    // cells from which forms 0-4 no longer hide the interface work, at that share of the
+    // cells, behind the liquid tiles of the same launch
+    long long shared_below = wide ? 1LL << 18 : 200000;
+    if (ifrac < 5) shared_below = wide ? 1LL << 23 : 1LL << 21;
+    if (ifrac < 3) shared_below = wide ? 1LL << 62 : 1LL << 24;
+    if (ifrac < 2) shared_below = 1LL << 62;
+    if (cells < shared_below) return FAM_SHARED;
+    if (wide) return !multi && cells >= 1LL << 20 && ifrac < 6 ? FAM_TWO : FAM_TILE;
+    return multi && cells >= 1LL << 23 ? FAM_TWO : FAM_TILE;
 }
+
+// A tuning decision holds for one shape of workload: storage precision, one or
+// many domains, SM count, lattice size (floor of log2 of the padded cells), the
+// interface cells among them (in 1/64) and the family the form is chosen from (0 in
+// FP64, where any form may be).
+struct TuneKey {
+    int prec, multi, sms, lsize, ifrac, family;
+    TuneKey(int prec_, bool multi_, int sms_, long long cells, long long interface_cells)
+        : prec(prec_), multi(multi_ ? 1 : 0), sms(sms_), lsize(0),
+          ifrac((int)(64 * interface_cells / (cells > 0 ? cells : 1))) {
+        while ((1LL << (lsize + 1)) <= cells) ++lsize;
+        family = prec == FSL_P_FP64 ? 0 : family_of(prec, multi_, cells, ifrac);
+    }
+    bool operator<(const TuneKey& o) const {
+        if (prec != o.prec) return prec < o.prec;
+        if (multi != o.multi) return multi < o.multi;
+        if (sms != o.sms) return sms < o.sms;
+        if (lsize != o.lsize) return lsize < o.lsize;
+        if (ifrac != o.ifrac) return ifrac < o.ifrac;
+        return family < o.family;
+    }
+};
 
 // The fastest measured form (ms: best time per form, 0 where it did not run) of
 // those the workload may run; usable[f]: form f can run on this handle now.
 inline int choose_form(const TuneKey& k, const double* ms, const bool* usable) {
     int best = -1, first = -1;
     for (int f = 0; f < SC_FORMS; ++f) {
-        if (!usable[f] || (k.prec != FSL_P_FP64 && form_family(f) != family_of(k))) continue;
+        if (!usable[f] || (k.prec != FSL_P_FP64 && form_family(f) != k.family)) continue;
         if (first < 0) first = f;
         if (ms[f] > 0.0 && (best < 0 || ms[f] < ms[best])) best = f;
     }
